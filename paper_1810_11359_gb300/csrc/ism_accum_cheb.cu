@@ -64,12 +64,12 @@ namespace {
 #define SH_B ISM_SHELL_BINS  // delay bins per CTA (a shell of 256 samples)
 #define SH_WARPS 8          // warps per CTA
 #define SH_NO 32            // offsets per bin (rr = -1 .. 30)
-#define SH_RS 33            // row stride of the moment table (conflict-light atomics)
+#define SH_RS (SH_B * SH_NO)   // row stride of the moment table: [term][bin, offset]
 #define CB_MAGIC 12582912.0f                       // 1.5 * 2^23
 static_assert(ISM_CHEB_NF == 8, "the expansion reads the moments as 4 + 4");
 // the expansion's moment table [bin][offset][8] overlays the sums, the counts, the scales, the
 // row prefix and the column records (all dead by then), which always span more than it needs
-static_assert(SH_B * SH_NO * 8 * 4 <= (SH_B * ISM_CHEB_NF * SH_RS + SH_B * SH_RS) * 4 + SH_WARPS * 32 * 32,
+static_assert(SH_B * SH_NO * 8 * 4 <= (ISM_CHEB_NF * SH_RS + SH_RS) * 4,
               "moment table larger than the tables it overlays");
 #define CB_MAGIC_BITS 0x4B400000u                  // its bits
 
@@ -103,24 +103,24 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
 
     // shared memory: axis tables | moment sums | image counts | per-bin scales | row prefix |
     // per-warp column records
-    float4* T = reinterpret_cast<float4*>(smem);
-    unsigned* S = reinterpret_cast<unsigned*>(smem + (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4));
-    int* Cn = reinterpret_cast<int*>(S + SH_B * ISM_CHEB_NF * SH_RS);             // [bin][offset] images
-    float* scale_s = reinterpret_cast<float*>(Cn + SH_B * SH_RS);
+    const ShellTab T = shell_tab(smem, t.max_axis_sum);
+    unsigned* S = reinterpret_cast<unsigned*>(smem + (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4));   // [term][bin, offset]
+    int* Cn = reinterpret_cast<int*>(S + ISM_CHEB_NF * SH_RS);                    // [bin, offset] images
+    float* scale_s = reinterpret_cast<float*>(Cn + SH_RS);
     float* inv_s = scale_s + SH_B;
     float* amax_s = inv_s + SH_B;                                                 // per-bin amplitude bound
     int* redo = reinterpret_cast<int*>(amax_s + SH_B);                            // [4]: retry flag
     int* rowpre = reinterpret_cast<int*>(redo + 4);                             // [Nx]: columns up to row ix
     int* rowy0 = rowpre + ((t.max_axis_sum + 4) & ~3);                          // [Nx]: first iy of row ix
     float4* recf = reinterpret_cast<float4*>(rowy0 + ((t.max_axis_sum + 4) & ~3));
-    int4* reci = reinterpret_cast<int4*>(recf + SH_WARPS * 32);
-    int* st = reinterpret_cast<int*>(reci + SH_WARPS * 32);                     // [warps][33]
+    int2* Wi = reinterpret_cast<int2*>(recf + SH_WARPS * 32) + warp * 32;
+    unsigned* Wm = reinterpret_cast<unsigned*>(Wi + (SH_WARPS - warp) * 32) + warp * SHELL_MW;   // [warps][SHELL_MW]
+    float* Wo = reinterpret_cast<float*>(Wm + (SH_WARPS - warp) * SHELL_MW) + warp * 32;  // [warps][32]: o_x D_x + o_y D_y
     float4* Wf = recf + warp * 32;
-    int4* Wi = reci + warp * 32;
-    int* Wst = st + warp * 33;
 
+    const float s2_magic = shell_s2_magic(J);
     const float4* Tg = tbl + J.tbl_base + (long long)r * n_axis;
-    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) T[e] = Tg[e];
+    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) shell_stage<true>(T, e, Tg[e], s2_magic);
     if (threadIdx.x == 0) *redo = 0;
     __syncthreads();
 
@@ -165,25 +165,21 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     }
     const int n_cols = shell_rows(sh, T, rowpre, rowy0);   // (synchronises the CTA)
 
-    const float amp_scale = J.amp_scale;
     for (int pass = 0; pass < 2; ++pass) {
-    for (int e = threadIdx.x; e < SH_B * ISM_CHEB_NF * SH_RS; e += blockDim.x) S[e] = 0;
-    for (int e = threadIdx.x; e < SH_B * SH_RS; e += blockDim.x) Cn[e] = 0;
+    for (int e = threadIdx.x; e < ISM_CHEB_NF * SH_RS; e += blockDim.x) S[e] = 0;
+    for (int e = threadIdx.x; e < SH_RS; e += blockDim.x) Cn[e] = 0;
     __syncthreads();
-    shell_walk<SH_WARPS>(sh, T, rowpre, rowy0, n_cols, make_float2(orient.x, orient.y), Wf, Wi, Wst, warp, lane,
-                         [&](int b, float f, float s, const float4& cf, int, int, const float4& tz) {
-        const int q = (b + 1) >> 5;
-        const int ql = q - q0;
-        const int o = b - ISM_SB * q + 1;   // offset index rr + 1 in [0, 32)
-        const float rs = ism_rcp(s);
-        float amp = cf.z * tz.z * amp_scale * rs;
+    shell_walk<SH_WARPS>(sh, T, rowpre, rowy0, n_cols, J.amp_scale, Wf, Wi, Wm, warp, lane, [&](int k, int ixy) {
+        if (alpha != 1.0f) Wo[k] = __fmaf_rn(orient.y, T.D(Nx + (ixy >> 16)), orient.x * T.D(ixy & 0xFFFF));
+    }, [&](int bl, float f, float rs, const float4& cf, int col, int, const float4& tz) {
+        float amp = cf.z * tz.z * rs;
         if (alpha != 1.0f)   // polar pattern: cos(theta) = o . (x_n - x_r) / d
-            amp *= __fmaf_rn(1.0f - alpha, __fmaf_rn(orient.z, tz.w, cf.w) * rs, alpha);
-        const float as = amp * scale_s[ql];
+            amp *= __fmaf_rn(1.0f - alpha, __fmaf_rn(orient.z, tz.w, Wo[col]) * rs, alpha);
+        const float as = amp * scale_s[bl >> 5];   // bin q0 + bl / 32, offset index rr + 1 = bl mod 32
         const float uu = __fmaf_rn(2.0f, f, -1.0f);
         const float u2 = uu + uu;
-        unsigned* Sb = S + ql * (ISM_CHEB_NF * SH_RS) + o;
-        atomicAdd(Cn + ql * SH_RS + o, 1);
+        unsigned* Sb = S + bl;
+        atomicAdd(Cn + bl, 1);
         atomicAdd(Sb, __float_as_uint(__fadd_rn(as, CB_MAGIC)));   // K + v: the n K go at the expansion
         atomicAdd(Sb + SH_RS, __float_as_uint(__fmaf_rn(as, uu, CB_MAGIC)));
         float tp = 1.0f, tc = uu;
@@ -201,7 +197,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     // the exact counts (the counts do not depend on the scales, so the second pass is safe)
     if (pass == 0 && threadIdx.x < SH_B) {
         int mx = 0;
-        for (int o = 0; o < SH_NO; ++o) mx = max(mx, Cn[threadIdx.x * SH_RS + o]);
+        for (int o = 0; o < SH_NO; ++o) mx = max(mx, Cn[threadIdx.x * SH_NO + o]);
         const float bound = (float)mx * (scale_s[threadIdx.x] * amax_s[threadIdx.x] + 0.5f);
         if (!(bound < 0.99f * 2147483648.0f)) {
             const float sc = shell_scale(amax_s[threadIdx.x], (float)mx);
@@ -218,12 +214,12 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     float m[ISM_CHEB_NF];
     bool any = false;
     if (warp < nb) {
-        const unsigned* Sb = S + warp * (ISM_CHEB_NF * SH_RS);
-        const unsigned nk = (unsigned)Cn[warp * SH_RS + lane] * CB_MAGIC_BITS;   // n K (mod 2^32)
+        const unsigned* Sb = S + warp * SH_NO + lane;
+        const unsigned nk = (unsigned)Cn[warp * SH_NO + lane] * CB_MAGIC_BITS;   // n K (mod 2^32)
         const float inv = inv_s[warp];
 #pragma unroll
         for (int k = 0; k < ISM_CHEB_NF; ++k) {
-            const int v = (int)(Sb[k * SH_RS + lane] - nk);
+            const int v = (int)(Sb[k * SH_RS] - nk);
             any |= v != 0;
             m[k] = __int2float_rn(v) * inv;   // exact scaling by a power of two
         }
@@ -262,10 +258,10 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
 
 size_t shell_smem(const JobTable& t)
 {
-    return (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4) + (size_t)SH_B * ISM_CHEB_NF * SH_RS * sizeof(int) +
-           (size_t)SH_B * SH_RS * sizeof(int) + 3 * SH_B * sizeof(float) + 4 * sizeof(int) +
-           2 * (size_t)((t.max_axis_sum + 4) & ~3) * sizeof(int) +
-           (size_t)SH_WARPS * 32 * (sizeof(float4) + sizeof(int4)) + (size_t)SH_WARPS * 33 * sizeof(int);
+    return (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4) + (size_t)(ISM_CHEB_NF + 1) * SH_RS * sizeof(int) +
+           3 * SH_B * sizeof(float) + 4 * sizeof(int) + 2 * (size_t)((t.max_axis_sum + 4) & ~3) * sizeof(int) +
+           (size_t)SH_WARPS * 32 * (sizeof(float4) + sizeof(int2)) +
+           (size_t)SH_WARPS * (SHELL_MW * sizeof(unsigned) + 32 * sizeof(float));
 }
 
 }  // namespace

@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
                                                                         float* __restrict__ rows, int winp)
 {
     constexpr bool HALF = PREC == PREC_FP16 || PREC == PREC_BF16;
+    constexpr bool SPLIT = PREC == PREC_FP32;   // squared offsets in split form (ism_shell.cuh)
     constexpr int LQ = ism_lut_phases(1);   // table phases per sample (LUT forms)
     constexpr int WIN = 64;   // window row of a bin: 32 (SLOTS + 1), SLOTS = 1
     extern __shared__ __align__(16) unsigned char smem[];
@@ -115,13 +116,15 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
 
     // shared memory: axis tables | row prefix | per-warp column records | per-warp staged
     // images | per-warp windows (winp floats each: the launch's thickest shell)
-    float4* T = reinterpret_cast<float4*>(smem);
+    const ShellTab T = shell_tab(smem, t.max_axis_sum);
     int* rowpre = reinterpret_cast<int*>(smem + (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4));
     int* rowy0 = rowpre + ((t.max_axis_sum + 4) & ~3);
     float4* recf = reinterpret_cast<float4*>(rowy0 + ((t.max_axis_sum + 4) & ~3));
-    int4* reci = reinterpret_cast<int4*>(recf + SD_WARPS * 32);
-    int* st = reinterpret_cast<int*>(reci + SD_WARPS * 32);                          // [warps][33]
-    float4* stage_all = reinterpret_cast<float4*>(st + SD_WARPS * 33 + 8);           // [warps][SD_RING]
+    int2* Wi = reinterpret_cast<int2*>(recf + SD_WARPS * 32);
+    unsigned* Wm = reinterpret_cast<unsigned*>(Wi + SD_WARPS * 32);                 // [warps][SHELL_MW]
+    float* Wo = reinterpret_cast<float*>(Wm + SD_WARPS * SHELL_MW);                   // [warps x 32]: o_x D_x + o_y D_y
+    unsigned char* Wb = reinterpret_cast<unsigned char*>(Wo + SD_WARPS * 32);         // [warps][SHELL_MW]
+    float4* stage_all = reinterpret_cast<float4*>(Wb + SD_WARPS * SHELL_MW);          // [warps][SD_RING]
     int* spos_all = reinterpret_cast<int*>(stage_all + SD_WARPS * SD_RING);           // [warps][SD_RING]
     int* wtot = spos_all + SD_WARPS * SD_RING;                                        // [warps]
     float* win_all = reinterpret_cast<float*>(wtot + SD_WARPS);                       // [warps][winp]
@@ -129,8 +132,9 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
     float4* stage = stage_all + warp * SD_RING;
     int* spos = spos_all + warp * SD_RING;
 
+    const float s2_magic = shell_s2_magic(J);
     const float4* Tg = tbl + J.tbl_base + (long long)r * n_axis;
-    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) T[e] = Tg[e];
+    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) shell_stage<SPLIT>(T, e, Tg[e], s2_magic);
     for (int w = 0; w < SD_WARPS; ++w)
         for (int e = threadIdx.x; e < win + 32; e += blockDim.x) win_all[w * winp + e] = 0.0f;
     __syncthreads();
@@ -168,10 +172,10 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
     const float f_hi = HALF ? 1.0f - 0x1p-13f : 1.0f;
     const float* lut = PREC == PREC_LUT ? lut_g + J.lut_base + lane : nullptr;
 
-    const int W0 = ISM_SB * q0 - 16;   // first sample of the shell's window
+    // (the shell's window starts at sample 32 q0 - 16: tap 0 of an image of integer delay
+    // 32 q0 - 1 + bl falls on its entry bl)
     const Shell sh = shell_setup(J, T, r, ISM_SB * q0 - 1, min(ISM_SB * (q0 + nb) - 1, J.n_ism + J.H - 1));
     const int n_cols = shell_rows(sh, T, rowpre, rowy0);   // (synchronises the CTA)
-    const float amp_scale = J.amp_scale;
 
     // Staged records: a ring of SD_RING per warp, records 2k and 2k + 1 interleaved as
     // {f_a, f_b, P_a, P_b}, {Pc_a, Pc_b, Ps_a, Ps_b}; the warp's images enter in the order
@@ -239,15 +243,17 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
         head = (head + n_pairs) & (SD_RING / 2 - 1);
     };
 
-    shell_walk_cta<SD_WARPS>(
-        sh, T, rowpre, rowy0, n_cols, make_float2(orient.x, orient.y), recf, reci, st, wtot, warp, lane,
-        [&](bool has, int b, float f, float s, const float4& cf, const float4& tz) {
+    shell_walk_cta<SD_WARPS, SPLIT>(
+        sh, T, rowpre, rowy0, n_cols, SPLIT ? J.amp_scale : 1.0f, recf, Wi, Wm, Wb, wtot, warp, lane,
+        [&](int k, int ixy) {
+            if (alpha != 1.0f) Wo[k] = __fmaf_rn(orient.y, T.D(Nx + (ixy >> 16)), orient.x * T.D(ixy & 0xFFFF));
+        },
+        [&](bool has, int bl, float f, float rs, const float4& cf, int col, int, const float4& tz) {
             float4 rc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (has) {
-                const float rs = ism_rcp(s);
-                float amp = cf.z * tz.z * amp_scale * rs;
+                float amp = SPLIT ? cf.z * tz.z * rs : cf.z * tz.z * J.amp_scale * rs;
                 if (alpha != 1.0f)   // polar pattern: cos(theta) = o . (x_n - x_r) / d
-                    amp *= __fmaf_rn(1.0f - alpha, __fmaf_rn(orient.z, tz.w, cf.w) * rs, alpha);
+                    amp *= __fmaf_rn(1.0f - alpha, __fmaf_rn(orient.z, tz.w, Wo[col]) * rs, alpha);
                 f = fminf(fmaxf(f, f_lo), f_hi);   // keeps j - f away from 0 (the reciprocal of the tap j = 0)
                 if constexpr (PREC == PREC_LUT) {
                     // eq. (9): rows floor(f Q) and + 1 of the polyphase table, weights A (1 - phi), A phi
@@ -266,7 +272,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
             }
             const unsigned v = __ballot_sync(0xffffffffu, has);
             if (has)   // the images of the batch in lane order, after those waiting
-                put((2 * head + n_st + __popc(v & ((1u << lane) - 1u))) & (SD_RING - 1), rc, b - 15 - W0);
+                put((2 * head + n_st + __popc(v & ((1u << lane) - 1u))) & (SD_RING - 1), rc, bl);
             n_st += __popc(v);
             if (n_st >= 32) {
                 __syncwarp();
@@ -319,7 +325,7 @@ int sd_bins_max(const JobTable& t)
 size_t shell_direct_smem(const JobTable& t)
 {
     return (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4) + 2 * (size_t)((t.max_axis_sum + 4) & ~3) * sizeof(int) +
-           (size_t)SD_WARPS * 32 * (sizeof(float4) + sizeof(int4)) + ((size_t)SD_WARPS * 33 + 8) * sizeof(int) +
+           (size_t)SD_WARPS * 32 * (sizeof(float4) + sizeof(int2) + sizeof(float)) + (size_t)SD_WARPS * SHELL_MW * (sizeof(unsigned) + 1) +
            (size_t)SD_WARPS * SD_RING * (sizeof(float4) + sizeof(int)) + SD_WARPS * sizeof(int) +
            (size_t)SD_WARPS * sd_winp(sd_bins_max(t)) * sizeof(float);
 }

@@ -57,21 +57,23 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     // shared memory: axis tables | derivative tables | Gamma tables | dLoss/dh windows |
     // warp sums | row prefix | per-warp column records
     const int axis_pad = (t.max_axis_sum + 1) & ~1;
-    float4* T = reinterpret_cast<float4*>(smem);
-    float4* X = T + axis_pad;                                   // x_n - x_r, dF/dbeta_lo, dF/dbeta_hi, d x_n / d x_s
+    const ShellTab T = shell_tab(smem, t.max_axis_sum);
+    float4* X = reinterpret_cast<float4*>(smem) + axis_pad;   // x_n - x_r, dF/dbeta_lo, dF/dbeta_hi, d x_n / d x_s
     float4* Gam = X + axis_pad;                                 // [bin][offset][SA_GV]: Gamma_0..8
     float* gw = reinterpret_cast<float*>(Gam + SA_B * 32 * SA_GV);   // [bin][64]
     float* red = gw + SA_B * 64;                                // [warp][SA_NG]
     int* rowpre = reinterpret_cast<int*>(red + SA_WARPS * SA_NG);
     int* rowy0 = rowpre + ((t.max_axis_sum + 4) & ~3);
     float4* recf = reinterpret_cast<float4*>(rowy0 + ((t.max_axis_sum + 4) & ~3));
-    int4* reci = reinterpret_cast<int4*>(recf + SA_WARPS * 32);
-    int* st = reinterpret_cast<int*>(reci + SA_WARPS * 32);     // [warps][33]
+    int2* Wi = reinterpret_cast<int2*>(recf + SA_WARPS * 32);
+    unsigned* Wm = reinterpret_cast<unsigned*>(Wi + SA_WARPS * 32);   // [warps][SHELL_MW]
+    int* Wx = reinterpret_cast<int*>(Wm + SA_WARPS * SHELL_MW) + warp * 32;   // [warps][32]: ix | iy << 16
 
+    const float s2_magic = shell_s2_magic(J);
     const float4* Tg = tbl + J.tbl_base + (long long)r * n_axis;
     const float4* Xg = dtbl + J.tbl_base + (long long)r * n_axis;
     for (int e = threadIdx.x; e < n_axis; e += blockDim.x) {
-        T[e] = Tg[e];
+        shell_stage<true>(T, e, Tg[e], s2_magic);
         X[e] = Xg[e];
     }
     // dLoss/dh over the windows of the CTA's bins (samples 32 q - 16 + P, P < 64; 0 outside [0, n_ism))
@@ -108,12 +110,10 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     for (int c = 0; c < SA_NG; ++c) G[c] = 0.0f;
     const float amp_scale = J.amp_scale;
     const float kfs = J.kfs_hi;   // f_s / c
-    shell_walk<SA_WARPS>(sh, T, rowpre, rowy0, n_cols, make_float2(0.0f, 0.0f), recf + warp * 32, reci + warp * 32,
-                         st + warp * 33, warp, lane,
-                         [&](int b, float f, float s, const float4& cf, int ixy, int iz, const float4& tz) {
-        const int q = (b + 1) >> 5;
-        const int o = b - ISM_SB * q + 1;   // offset index rr + 1 in [0, 32)
-        const float4* Gr = Gam + ((q - q0) * 32 + o) * SA_GV;
+    shell_walk<SA_WARPS>(sh, T, rowpre, rowy0, n_cols, 1.0f, recf + warp * 32, Wi + warp * 32, Wm + warp * SHELL_MW, warp, lane,
+                         [&](int k, int ixy) { Wx[k] = ixy; },
+                         [&](int bl, float f, float rs, const float4& cf, int col, int ez, const float4& tz) {
+        const float4* Gr = Gam + bl * SA_GV;   // [bin][offset], 32 offsets per bin
         const float4 g0 = Gr[0], g1 = Gr[1], g2 = Gr[2];
         const float Gb[ISM_CHEB_N] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w, g2.x};
         // ga = sum_i Gamma_i T_i(u), gd = sum_i Gamma_i T_i'(u)
@@ -134,11 +134,11 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
             dp = dc;
             dc = dn;
         }
-        const int ix = ixy & 0xFFFF, iy = ixy >> 16;
-        const float4 tx = T[ix], ty = T[Nx + iy];
-        const float4 xx = X[ix], xy = X[Nx + iy], xz = X[Nx + Ny + iz];
-        const float rs = ism_rcp(s);
-        const float A = cf.z * tz.z * amp_scale * rs;        // eq. (4), as in the forward
+        const int ex = Wx[col] & 0xFFFF, ey = Nx + (Wx[col] >> 16);
+        const float4 xx = X[ex], xy = X[ey], xz = X[ez];
+        const float4 tx = T.all(ex), ty = T.all(ey);
+        const float Fx = tx.z, Fy = ty.z, Fz = tz.z;
+        const float A = cf.z * Fz * amp_scale * rs;        // eq. (4), as in the forward
         // c = -(A / d) ga - (f_s / c) A ge with 1 / d = (f_s / c) / s and ge = -2 gd
         const float cr = A * kfs * __fmaf_rn(2.0f, gd, -rs * ga) * rs;
         // (p_r - p_n) / d = -D / s per axis (D = signed offset in samples)
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
         G[4] = __fmaf_rn(cr, xy.w * ty.w, G[4]);
         G[5] = __fmaf_rn(cr, xz.w * tz.w, G[5]);
         const float gs = ga * amp_scale * rs;                // ga / (4 pi d)
-        const float Fyz = ty.z * tz.z, Fxz = tx.z * tz.z, Fxy = cf.z;
+        const float Fyz = Fy * Fz, Fxz = Fx * Fz, Fxy = cf.z;
         G[6] = __fmaf_rn(gs, xx.y * Fyz, G[6]);
         G[7] = __fmaf_rn(gs, xx.z * Fyz, G[7]);
         G[8] = __fmaf_rn(gs, xy.y * Fxz, G[8]);
@@ -182,7 +182,7 @@ size_t shell_adjoint_smem(const JobTable& t)
     const size_t rows = (size_t)((t.max_axis_sum + 4) & ~3);
     return 2 * axis_pad * sizeof(float4) + (size_t)SA_B * 32 * SA_GV * sizeof(float4) +
            (size_t)SA_B * 64 * sizeof(float) + (size_t)SA_WARPS * SA_NG * sizeof(float) + 2 * rows * sizeof(int) +
-           (size_t)SA_WARPS * 32 * (sizeof(float4) + sizeof(int4)) + (size_t)SA_WARPS * 33 * sizeof(int);
+           (size_t)SA_WARPS * 32 * (sizeof(float4) + sizeof(int2) + sizeof(int)) + (size_t)SA_WARPS * SHELL_MW * sizeof(unsigned);
 }
 
 }  // namespace
