@@ -1,6 +1,7 @@
-// ism_accum_cheb.cu -- FP32 accumulation of eq. (5) for a 32-tap window
-// through a Chebyshev expansion of the windowed sinc in the fractional delay,
-// fused with the enumeration of the images (Section 2.1) it accumulates.
+// ism_accum_cheb.cu -- FP32 accumulation of eq. (5) through a Chebyshev
+// expansion of the windowed sinc in the fractional delay, fused with the
+// enumeration of the images (Section 2.1) it accumulates: 32-tap windows with
+// 8 terms (the text below), other windows of 16 taps or more with 10.
 //
 // For tap j of an image with delay s = b + f (b integer, f in [0, 1)), the
 // sample b + j receives A delta'(j - f) (eq. (6)).  For a window of exactly
@@ -56,44 +57,61 @@
 // (lane = tap) and rotates them into the bin's register window, which it
 // stores as the bin's row; the moments of an offset sit together (8 floats),
 // so a warp reads them in two broadcast loads.
+//
+// Other windows (the default, 4 ms, is 64 taps at 16 kHz and 176.4 at 44.1 kHz).
+// A window whose end falls inside a sample interval cuts its last taps with a
+// mask, which no polynomial follows, but the window has a double zero there:
+// for 16 taps or more the kink is below 2.7e-8 of the amplitude and degree 9
+// reproduces every tap to that (2.5e-9 without a mask).  The 2 H coefficients
+// of each term come from a table in the workspace that the geometry launch
+// fills (cheb_table), and the expansion takes 32 taps at a time, each turn's
+// upper half carried into the next.  The terms are converted to integers
+// (cvt.rni) instead of rounded by the FFMA, which lifts the 2^22 cap on a
+// term: with few images per integer delay the sums then hold up to 30 bits of
+// a term, and a sparse RIR's error stays at the per-tap sum's (3.6e-7 of its
+// norm with the cap, 1.6e-7 without it, 1.4e-7 per tap, 15 RIRs of 176 taps),
+// at no cost in time (the conversions go to a unit that is 14 % busy).
 #include "ism_accum.cuh"
 #include "ism_shell.cuh"
 
 namespace {
 
-#define SH_B ISM_SHELL_BINS  // delay bins per CTA (a shell of 256 samples)
+#define SH_B ISM_SHELL_BINS  // delay bins per CTA (a shell of 256 samples), fewer for small launches
 #define SH_WARPS 8          // warps per CTA
+#define SH_RS (SH_B * 32)   // row stride of the moment table: [term][bin, offset]
 #define SH_NO 32            // offsets per bin (rr = -1 .. 30)
-#define SH_RS (SH_B * SH_NO)   // row stride of the moment table: [term][bin, offset]
 #define CB_MAGIC 12582912.0f                       // 1.5 * 2^23
-static_assert(ISM_CHEB_NF == 8, "the expansion reads the moments as 4 + 4");
-// the expansion's moment table [bin][offset][8] overlays the sums, the counts, the scales, the
-// row prefix and the column records (all dead by then), which always span more than it needs
-static_assert(SH_B * SH_NO * 8 * 4 <= (ISM_CHEB_NF * SH_RS + SH_RS) * 4,
-              "moment table larger than the tables it overlays");
 #define CB_MAGIC_BITS 0x4B400000u                  // its bits
 
-// Largest power of two 2^e with 2^e a_max <= min((1 - 2^-10) 2^22, 0.98 2^31 / n - 1):
-// no term reaches 2^22 (the FFMA rounding trick) and n terms cannot sum to 2^31.
-__device__ __forceinline__ float shell_scale(float a_max, float n)
+// Largest power of two 2^e with 2^e a_max <= min((1 - 2^-10) term_max, 0.98 2^31 / n - 1):
+// no term reaches term_max (2^22 with the FFMA rounding trick) and n terms cannot sum to 2^31.
+__device__ __forceinline__ float shell_scale(float a_max, float n, float term_max)
 {
-    const float cap = fminf(4194304.0f * (1.0f - 1.0f / 1024.0f), 0.98f * 2147483648.0f / fmaxf(n, 1.0f) - 1.0f);
+    const float cap = fminf(term_max * (1.0f - 1.0f / 1024.0f), 0.98f * 2147483648.0f / fmaxf(n, 1.0f) - 1.0f);
     const float ratio = a_max > 0.0f ? cap / a_max : 3.0e38f;
     int e = ((__float_as_int(ratio) >> 23) & 0xFF) - 127;   // floor(log2(ratio)), ratio normal
     e = max(-126, min(126, e));
     return __int_as_float((e + 127) << 23);
 }
 
+template <int NM>
 __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_constant__ JobTable t,
                                                                   const float4* __restrict__ tbl,
-                                                                  float* __restrict__ rows,
-                                                                  uint32_t* __restrict__ status)
+                                                                  const float* __restrict__ tabs,
+                                                                  float* __restrict__ rows)
 {
-    constexpr int WIN = 64;   // 32 (SLOTS + 1), SLOTS = 1
+    constexpr float TERM_MAX = NM != ISM_CHEB_NF ? 1073741824.0f : 4194304.0f;
+    constexpr bool CVT = NM != ISM_CHEB_NF;   // terms converted to integers, not rounded by the FFMA
+    constexpr int MV = (NM + 3) / 4;   // float4 per offset of the expansion's moment table
+    // [bin][offset][4 MV], which overlays the sums, the counts, the scales, the row prefix and
+    // the column records (all dead by then)
+    static_assert(SH_RS * MV * 16 <= (NM + 1) * SH_RS * 4 + SH_WARPS * 32 * 24,
+                  "moment table larger than the tables it overlays");
     extern __shared__ __align__(16) unsigned char smem[];
     int jid, r, grp;
     if (!shell_cta(t, blockIdx.x, &jid, &r, &grp)) return;   // CTA-uniform
     const JobDev& J = t.j[jid];
+    if (J.use_cheb != NM) return;   // another instantiation's job
     const int B = t.shell_bins;   // bins of this launch's shells: SH_B, fewer for small launch sets
     const int q0 = grp * B;
     const int nb = min(B, J.Q - q0);
@@ -105,7 +123,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     // per-warp column records
     const ShellTab T = shell_tab(smem, t.max_axis_sum);
     unsigned* S = reinterpret_cast<unsigned*>(smem + (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4));   // [term][bin, offset]
-    int* Cn = reinterpret_cast<int*>(S + ISM_CHEB_NF * SH_RS);                    // [bin, offset] images
+    int* Cn = reinterpret_cast<int*>(S + NM * SH_RS);                    // [bin, offset] images
     float* scale_s = reinterpret_cast<float*>(Cn + SH_RS);
     float* inv_s = scale_s + SH_B;
     float* amax_s = inv_s + SH_B;                                                 // per-bin amplitude bound
@@ -157,7 +175,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
             const float k = 1.0f / kinv;
             const float vol = J.vol;
             const float n_est = 4.0f * (12.566371f * shi * shi / (k * k * k * vol)) + 64.0f;
-            sc = shell_scale(amax, n_est);
+            sc = shell_scale(amax, n_est, TERM_MAX);
         }
         scale_s[threadIdx.x] = sc;
         inv_s[threadIdx.x] = 1.0f / sc;   // exact: a power of two
@@ -166,7 +184,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     const int n_cols = shell_rows(sh, T, rowpre, rowy0);   // (synchronises the CTA)
 
     for (int pass = 0; pass < 2; ++pass) {
-    for (int e = threadIdx.x; e < ISM_CHEB_NF * SH_RS; e += blockDim.x) S[e] = 0;
+    for (int e = threadIdx.x; e < NM * SH_RS; e += blockDim.x) S[e] = 0;
     for (int e = threadIdx.x; e < SH_RS; e += blockDim.x) Cn[e] = 0;
     __syncthreads();
     shell_walk<SH_WARPS>(sh, T, rowpre, rowy0, n_cols, J.amp_scale, Wf, Wi, Wm, warp, lane, [&](int k, int ixy) {
@@ -180,13 +198,17 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
         const float u2 = uu + uu;
         unsigned* Sb = S + bl;
         atomicAdd(Cn + bl, 1);
-        atomicAdd(Sb, __float_as_uint(__fadd_rn(as, CB_MAGIC)));   // K + v: the n K go at the expansion
-        atomicAdd(Sb + SH_RS, __float_as_uint(__fmaf_rn(as, uu, CB_MAGIC)));
+        // the term's bits in the sum: K + v by the FFMA trick (the n K go at the expansion), or v
+        auto term = [&](float tk) {
+            return CVT ? (unsigned)__float2int_rn(as * tk) : __float_as_uint(__fmaf_rn(as, tk, CB_MAGIC));
+        };
+        atomicAdd(Sb, CVT ? (unsigned)__float2int_rn(as) : __float_as_uint(__fadd_rn(as, CB_MAGIC)));
+        atomicAdd(Sb + SH_RS, term(uu));
         float tp = 1.0f, tc = uu;
 #pragma unroll
-        for (int k = 2; k < ISM_CHEB_NF; ++k) {
+        for (int k = 2; k < NM; ++k) {
             const float tn = __fmaf_rn(u2, tc, -tp);
-            atomicAdd(Sb + k * SH_RS, __float_as_uint(__fmaf_rn(as, tn, CB_MAGIC)));
+            atomicAdd(Sb + k * SH_RS, term(tn));
             tp = tc;
             tc = tn;
         }
@@ -200,7 +222,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
         for (int o = 0; o < SH_NO; ++o) mx = max(mx, Cn[threadIdx.x * SH_NO + o]);
         const float bound = (float)mx * (scale_s[threadIdx.x] * amax_s[threadIdx.x] + 0.5f);
         if (!(bound < 0.99f * 2147483648.0f)) {
-            const float sc = shell_scale(amax_s[threadIdx.x], (float)mx);
+            const float sc = shell_scale(amax_s[threadIdx.x], (float)mx, TERM_MAX);
             scale_s[threadIdx.x] = sc;
             inv_s[threadIdx.x] = 1.0f / sc;
             atomicOr(redo, 1);
@@ -211,57 +233,79 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     }
 
     // ---- expansion: warp w owns bin q0 + w; lane o reads the sums of offset o
-    float m[ISM_CHEB_NF];
+    float m[4 * MV];
     bool any = false;
     if (warp < nb) {
         const unsigned* Sb = S + warp * SH_NO + lane;
-        const unsigned nk = (unsigned)Cn[warp * SH_NO + lane] * CB_MAGIC_BITS;   // n K (mod 2^32)
+        // n K (mod 2^32) of the biased terms
+        const unsigned nk = CVT ? 0u : (unsigned)Cn[warp * SH_NO + lane] * CB_MAGIC_BITS;
         const float inv = inv_s[warp];
 #pragma unroll
-        for (int k = 0; k < ISM_CHEB_NF; ++k) {
-            const int v = (int)(Sb[k * SH_RS] - nk);
+        for (int k = 0; k < 4 * MV; ++k) {
+            const int v = k < NM ? (int)(Sb[k * SH_RS] - nk) : 0;
             any |= v != 0;
             m[k] = __int2float_rn(v) * inv;   // exact scaling by a power of two
         }
     }
     __syncthreads();   // every sum is read before the moment table overwrites the CTA's tables
     if (warp >= nb) return;
-    const int q = q0 + warp;
-    // moments of (bin, offset o) at Mt + 2 (32 bin + o): {M_0..M_3}, {M_4..M_7}
-    float4* Mt = reinterpret_cast<float4*>(S);
-    {
-        float4* mo = Mt + 2 * (32 * warp + lane);
-        mo[0] = make_float4(m[0], m[1], m[2], m[3]);
-        mo[1] = make_float4(m[4], m[5], m[6], m[7]);
-    }
+    // moments of (bin, offset o) at Mt + MV (32 bin + o): {M_0..M_3}, {M_4..M_7}, ..
+    float4* Mt = reinterpret_cast<float4*>(S) + MV * SH_NO * warp;
+#pragma unroll
+    for (int v = 0; v < MV; ++v) Mt[MV * lane + v] = make_float4(m[4 * v], m[4 * v + 1], m[4 * v + 2], m[4 * v + 3]);
     const unsigned nonempty = __ballot_sync(0xffffffffu, any);
     __syncwarp();
-    float c[ISM_CHEB_NF];   // lane = tap t: Chebyshev coefficients of g_(t - 15)
+    const int slots = NM == ISM_CHEB_NF ? 1 : J.slots;
+    float* row = rows + J.rows_base + ((long long)r * J.Q + q0 + warp) * (32 * (slots + 1));
+    float carry = 0.0f;   // the previous 32 taps' share of this 32 samples
+    for (int sl = 0; sl < slots; ++sl) {
+        float c[NM];   // lane = tap 32 sl + lane: its Chebyshev coefficients
 #pragma unroll
-    for (int i = 0; i < ISM_CHEB_NF; ++i) c[i] = t.cheb[lane * ISM_CHEB_N + i];
-    float acc[2] = {0.0f, 0.0f};
-    for (int o = 0; o < SH_NO; ++o) {
-        if (!((nonempty >> o) & 1u)) continue;   // warp-uniform
-        const float4* mo = Mt + 2 * (32 * warp + o);
-        const float4 ma = mo[0], mb = mo[1];
-        const float mv[ISM_CHEB_NF] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
-        float D[1];
-        D[0] = c[0] * mv[0];
+        for (int i = 0; i < NM; ++i)
+            c[i] = NM == ISM_CHEB_NF ? t.cheb[lane * ISM_CHEB_N + i] : tabs[J.lut_base + (i * slots + sl) * 32 + lane];
+        float acc[2] = {carry, 0.0f};
+        for (int o = 0; o < SH_NO; ++o) {
+            if (!((nonempty >> o) & 1u)) continue;   // warp-uniform
+            float mv[4 * MV];
 #pragma unroll
-        for (int k = 1; k < ISM_CHEB_NF; ++k) D[0] = __fmaf_rn(c[k], mv[k], D[0]);
-        flush_run<1, false>(D, acc, o - 1, lane, 1.0f);
+            for (int v = 0; v < MV; ++v) {
+                const float4 w = Mt[MV * o + v];
+                mv[4 * v] = w.x;
+                mv[4 * v + 1] = w.y;
+                mv[4 * v + 2] = w.z;
+                mv[4 * v + 3] = w.w;
+            }
+            float D[1];
+            D[0] = c[0] * mv[0];
+#pragma unroll
+            for (int k = 1; k < NM; ++k) D[0] = __fmaf_rn(c[k], mv[k], D[0]);
+            flush_run<1, false>(D, acc, o - 1, lane, 1.0f);
+        }
+        row[32 * sl + lane] = acc[0];
+        carry = acc[1];
     }
-    float* row = rows + J.rows_base + ((long long)r * J.Q + q) * WIN;
-    row[lane] = acc[0];
-    row[32 + lane] = acc[1];
+    row[32 * slots + lane] = carry;
 }
 
-size_t shell_smem(const JobTable& t)
+template <int NM>
+int launch_cheb(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s, int* launched)
 {
-    return (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4) + (size_t)(ISM_CHEB_NF + 1) * SH_RS * sizeof(int) +
-           3 * SH_B * sizeof(float) + 4 * sizeof(int) + 2 * (size_t)((t.max_axis_sum + 4) & ~3) * sizeof(int) +
-           (size_t)SH_WARPS * 32 * (sizeof(float4) + sizeof(int2)) +
-           (size_t)SH_WARPS * (SHELL_MW * sizeof(unsigned) + 32 * sizeof(float));
+    const size_t sm = (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4) + (size_t)(NM + 1) * SH_RS * sizeof(int) +
+                      3 * SH_B * sizeof(float) + 4 * sizeof(int) + 2 * (size_t)((t.max_axis_sum + 4) & ~3) * sizeof(int) +
+                      (size_t)SH_WARPS * 32 * (sizeof(float4) + sizeof(int2)) +
+                      (size_t)SH_WARPS * (SHELL_MW * sizeof(unsigned) + 32 * sizeof(float));
+    static std::atomic<unsigned long long> opened{0};
+    int rc = ism_open_smem((const void*)shell_kernel<NM>, &opened);
+    if (rc) return rc;
+    // all of the unified L1 as shared memory: 5 CTAs of ~27 KB per SM
+    cudaError_t e = cudaFuncSetAttribute(shell_kernel<NM>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return (int)e;
+    shell_kernel<NM><<<(unsigned)p.shell_ctas, SH_WARPS * 32, sm, s>>>(
+        t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<const float*>(ws + p.lut_off),
+        reinterpret_cast<float*>(ws + p.rows_off));
+    ++*launched;
+    return (int)cudaGetLastError();
 }
 
 }  // namespace
@@ -270,17 +314,14 @@ int ism_launch_accum_cheb(const JobTable& t, const WsPlan& p, char* ws, void* st
 {
     *launched = 0;
     if (p.shell_ctas <= 0 || !t.any_cheb) return 0;
-    const size_t sm = shell_smem(t);
-    static std::atomic<unsigned long long> opened{0};
-    int rc = ism_open_smem((const void*)shell_kernel, &opened);
-    if (rc) return rc;
-    // all of the unified L1 as shared memory: 5 CTAs of ~27 KB per SM
-    cudaError_t e = cudaFuncSetAttribute(shell_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return (int)e;
-    shell_kernel<<<(unsigned)p.shell_ctas, SH_WARPS * 32, sm, (cudaStream_t)stream>>>(
-        t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<float*>(ws + p.rows_off),
-        reinterpret_cast<uint32_t*>(ws + p.status_off));
-    *launched = 1;
-    return (int)cudaGetLastError();
+    bool plain = false, wide = false;
+    for (int i = 0; i < t.n_jobs; ++i) {
+        plain |= t.j[i].use_cheb == ISM_CHEB_NF;
+        wide |= t.j[i].use_cheb == ISM_CHEB_NW;
+    }
+    int rc = 0;
+    cudaStream_t s = (cudaStream_t)stream;
+    if (plain) rc = launch_cheb<ISM_CHEB_NF>(t, p, ws, s, launched);
+    if (!rc && wide) rc = launch_cheb<ISM_CHEB_NW>(t, p, ws, s, launched);
+    return rc;
 }

@@ -166,8 +166,10 @@ const float* cheb_coefficients(bool forward)
 
 // Lays the launch set out in the workspace from byte offset `base` on (the
 // status word is always at offset 0, shared by every launch set of a call).
+// binned: as if FP32 windows of other than 32 taps went through binned image
+// ids (sizes only: the allocation-free entry point's limit counts them).
 ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, JobTable& t, WsPlan& p,
-                size_t base = 0)
+                size_t base = 0, bool binned = false)
 {
     std::memset(&t, 0, sizeof t);
     std::memset(&p, 0, sizeof p);
@@ -284,8 +286,18 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
             const double in_reach = std::min((double)in.nb_img[0] * in.nb_img[1] * in.nb_img[2],
                                              4.18879020478639 * reach * reach * reach / vol);
             const double per_bin = in_reach / (double)((v.n_ism + v.H) / ISM_SB + 1);
-            J.use_cheb = (prec == ISM_PREC_FP32 && !backward && v.Nw == 32.0 && v.H == 16 && v.slots == 1 &&
-                          per_bin >= 64.0) ? 1 : 0;
+            // Other windows take them from 20 images per bin on, at degree 9, whose series keeps
+            // the per-tap sum's accuracy for every window of ISM_CHEB_MIN_NW taps or more: the
+            // form they take below that has passes over the images to count, scan and scatter
+            // before it.  Measured against it (a call, us): 16 RIRs of 64 taps, 5500 per bin,
+            // 2000 -> 350; of 176 taps, 27 per bin, 15 RIRs 63 -> 42 and 512 RIRs 450 -> 415;
+            // 6 per bin, 512 RIRs 122 -> 151; of 40 taps, 43 per bin, 512 RIRs 445 -> 329; 11
+            // per bin, 131 -> 133.
+            const bool taps32 = v.Nw == 32.0;
+            J.use_cheb = 0;
+            if (prec == ISM_PREC_FP32 && !backward && taps32 && per_bin >= 64.0) J.use_cheb = ISM_CHEB_NF;
+            if (prec == ISM_PREC_FP32 && !backward && !taps32 && per_bin >= 20.0 && v.Nw >= ISM_CHEB_MIN_NW && !binned)
+                J.use_cheb = ISM_CHEB_NW;
             // sparse bins: sorting by offset and padding each offset to a group of 4
             // images costs more than adding every image's taps on its own
             J.sparse = ((prec == ISM_PREC_FP32 || prec == ISM_PREC_FP32_DIRECT) && !backward && !J.use_cheb &&
@@ -296,8 +308,7 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
             // the other forward jobs with a 32-tap window, in every tap arithmetic: every tap
             // evaluated, the images enumerated by the CTA that accumulates them (no ids, no
             // sort); the value is the shell's thickness in bins: 32 for sparse bins, 8 for dense ones
-            J.shell_direct = (!backward && !J.use_cheb && v.Nw == 32.0 && v.H == 16 && v.slots == 1)
-                                 ? (per_bin < 64.0 ? ISM_SD_BINS : 8) : 0;
+            J.shell_direct = (!backward && !J.use_cheb && taps32) ? (per_bin < 64.0 ? ISM_SD_BINS : 8) : 0;
         }
         const bool cheb = J.use_cheb || J.adj_cheb;
         const bool fused = cheb || J.shell_direct;
@@ -355,6 +366,18 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
         if (prec == ISM_PREC_LUT) lut += (long long)(ism_lut_phases(J.slots) + 1) * 32 * J.slots;
         // texture form: each table starts on a 512-byte boundary (texture base alignment)
         if (prec == ISM_PREC_LUT_TEX) lut += ((long long)(ism_lut_phases(J.slots) + 1) * 32 * J.slots + 127) / 128 * 128;
+        if (J.use_cheb == ISM_CHEB_NW) {   // one coefficient table per window length
+            J.lut_base = p.cheb_tabs * ISM_CHEB_TAB;
+            for (int k = 0; k < i; ++k)
+                if (t.j[k].use_cheb == J.use_cheb && t.j[k].Nw == J.Nw) {
+                    J.lut_base = t.j[k].lut_base;
+                    break;
+                }
+            if (J.lut_base == p.cheb_tabs * ISM_CHEB_TAB) {
+                ++p.cheb_tabs;
+                lut += ISM_CHEB_TAB;
+            }
+        }
         if (cheb) t.any_cheb = 1;
         else if (!fused) t.any_direct = 1;
         if (backward) gpart += R * J.Q * 12;
@@ -549,20 +572,21 @@ Schedule schedule(const std::vector<Validated>& vs)
 
 // Workspace of a schedule: lane 0's sets reuse [0, base1), lane 1's sets
 // [base1, need); *base1_out receives base1.
-ism_status schedule_size(const Schedule& sc, ism_precision prec, size_t* bytes, size_t* base1_out)
+ism_status schedule_size(const Schedule& sc, ism_precision prec, size_t* bytes, size_t* base1_out,
+                         bool binned = false)
 {
     JobTable t;
     WsPlan p;
     size_t size0 = 256, size1 = 0;
     for (size_t k = 0; k < sc.sets.size(); k += sc.lanes) {
-        ism_status s = plan(sc.sets[k].data(), (int)sc.sets[k].size(), prec, false, t, p, 0);
+        ism_status s = plan(sc.sets[k].data(), (int)sc.sets[k].size(), prec, false, t, p, 0, binned);
         if (s != ISM_OK) return s;
         size0 = std::max(size0, p.total);
     }
     const size_t base1 = align256(size0);
     if (sc.lanes == 2)
         for (size_t k = 1; k < sc.sets.size(); k += 2) {
-            ism_status s = plan(sc.sets[k].data(), (int)sc.sets[k].size(), prec, false, t, p, base1);
+            ism_status s = plan(sc.sets[k].data(), (int)sc.sets[k].size(), prec, false, t, p, base1, binned);
             if (s != ISM_OK) return s;
             size1 = std::max(size1, p.total - base1);
         }
@@ -830,7 +854,7 @@ ism_status run_set(const std::vector<Validated>& set, ism_precision prec, size_t
     {
         StageTimer tm(ISM_STAGE_ACCUM, st);
         int launched = 0;
-        if (p.lut_total > 0) {
+        if (p.lut_total > 0 && !p.cheb_tabs) {   // (Chebyshev coefficients come from the geometry launch)
             if ((e = ism_launch_lut_tables(t, p, ws, stream))) return cuda_fail(e, "windowed-sinc table kernel");
             ++launched;
         }
@@ -1760,7 +1784,9 @@ extern "C" ism_status ism_simulate_noalloc(const ism_room* room, const float* po
     std::vector<Validated> vs;
     if ((s = validate_all(&j, 1, vs, true)) != ISM_OK) return s;
     size_t need = 0;
-    if ((s = batch_size(vs, prec, &need)) != ISM_OK) return s;
+    // (the limit counts the scratch of binned image ids, whichever kernels take the call: what
+    // it admits does not change with them, and the fused forms need less)
+    if ((s = schedule_size(schedule(vs), prec, &need, nullptr, true)) != ISM_OK) return s;
     if (need > ISM_NOALLOC_SCRATCH_BYTES)
         return fail(ISM_ERR_UNSUPPORTED,
                     "this simulation needs %zu bytes of scratch, above the %u bytes of the allocation-free "

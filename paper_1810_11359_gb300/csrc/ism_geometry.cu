@@ -34,9 +34,49 @@ __device__ double dpow_int(double b, int e)
     return r;
 }
 
-__global__ void __launch_bounds__(128) geometry_kernel(const __grid_constant__ JobTable t, float4* tbl,
-                                                       float4* dtbl, uint32_t* status)
+// Chebyshev coefficients of 8 of the tap functions g_t(f) = delta'(t - H + 1 - f) (eq. (6))
+// of a window of N_w taps, f = (u + 1) / 2: interpolated at the Chebyshev-Gauss nodes
+// u_k = cos(pi (k + 1/2) / N), c_i = (2 / N) sum_k g_t(u_k) T_i(u_k), c_0 halved, in FP64.
+// (GB300's FP64 pipe is narrow: 8 taps per CTA spread the ~100 values a tap over the SMs
+// beside the geometry CTAs, which take longer.)
+__device__ void cheb_table(const JobDev& J, int N, int tap0, float* tab)
 {
+    __shared__ double gv[8][ISM_CHEB_MAX], cs[ISM_CHEB_MAX][ISM_CHEB_MAX];   // g_t(u_k); T_i(u_k)
+    for (int e = threadIdx.x; e < 8 * N; e += blockDim.x) {
+        const int k = e % N, t = tap0 + e / N;
+        const double f = 0.5 * (cospi((k + 0.5) / N) + 1.0);
+        const int j = t - J.H + 1;
+        const double x = (double)j - f, Nw = (double)J.Nw;
+        double v = 0.0;
+        if (t < 2 * J.H && fabs(x) < 0.5 * Nw)   // sin(pi (j - f)) = (-1)^(j + 1) sin(pi f)
+            v = 0.5 * (1.0 + cospi(2.0 * x / Nw)) * ((j & 1) ? 1.0 : -1.0) * sinpi(f) /
+                (3.141592653589793238462643383279502884 * x);
+        gv[e / N][k] = v;
+    }
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) cs[e / N][e % N] = cospi((e / N) * (e % N + 0.5) / N);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 8 * N; e += blockDim.x) {
+        const int i = e / 8, t = tap0 + e % 8;
+        double c = 0.0;
+        for (int k = 0; k < N; ++k) c += gv[e % 8][k] * cs[i][k];
+        tab[i * 32 * J.slots + t] = (float)(c * (i == 0 ? 1.0 : 2.0) / N);
+    }
+}
+
+__global__ void __launch_bounds__(128) geometry_kernel(const __grid_constant__ JobTable t, float4* tbl,
+                                                       float4* dtbl, uint32_t* status, float* tabs, int n_rir)
+{
+    if ((int)blockIdx.x >= n_rir) {   // the coefficient tables: ISM_CHEB_TAB_CTAS CTAs each
+        const int k = ((int)blockIdx.x - n_rir) / ISM_CHEB_TAB_CTAS, c = ((int)blockIdx.x - n_rir) % ISM_CHEB_TAB_CTAS;
+        for (int i = 0; i < t.n_jobs; ++i) {
+            const JobDev& J = t.j[i];
+            const int N = J.use_cheb > J.adj_cheb ? J.use_cheb : J.adj_cheb;
+            if (N < ISM_CHEB_NW || J.lut_base != k * ISM_CHEB_TAB) continue;
+            if (8 * c < 32 * J.slots) cheb_table(J, N, 8 * c, tabs + J.lut_base);
+            return;
+        }
+        return;
+    }
     const long long g = blockIdx.x;  // one CTA per RIR of the launch set
     const int jid = ism_find_job(t, g, [](const JobDev& j) { return j.rir_base; });
     const JobDev& J = t.j[jid];
@@ -146,9 +186,9 @@ int ism_launch_geometry(const JobTable& t, const WsPlan& p, char* ws, void* stre
 {
     long long n_rir = p.rir_total;
     if (n_rir <= 0) return 0;
-    geometry_kernel<<<(unsigned)n_rir, 128, 0, (cudaStream_t)stream>>>(
+    geometry_kernel<<<(unsigned)(n_rir + ISM_CHEB_TAB_CTAS * p.cheb_tabs), 128, 0, (cudaStream_t)stream>>>(
         t, reinterpret_cast<float4*>(ws + p.tbl_off), p.dtbl_off ? reinterpret_cast<float4*>(ws + p.dtbl_off) : nullptr,
-        reinterpret_cast<uint32_t*>(ws + p.status_off));
+        reinterpret_cast<uint32_t*>(ws + p.status_off), reinterpret_cast<float*>(ws + p.lut_off), (int)n_rir);
     return (int)cudaGetLastError();
 }
 

@@ -46,6 +46,11 @@
 #define ISM_FIT_WINDOW_S 0.02     // envelope fit: last 20 ms of the ISM part
 #define ISM_CHEB_N 9              // Chebyshev terms of a tap function in the adjoint (degree 8); table stride
 #define ISM_CHEB_NF 8             // Chebyshev terms of the forward's moments (degree 7)
+#define ISM_CHEB_NW 10            // the same for windows other than 32 taps (degree 9)
+#define ISM_CHEB_MIN_NW 16        // shortest window whose taps the series reproduces (see ism_accum_cheb.cu)
+#define ISM_CHEB_MAX 12           // terms of any of them, at most
+#define ISM_CHEB_TAB 4096         // floats of a coefficient table in the workspace: [term][32 slots]
+#define ISM_CHEB_TAB_CTAS 32      // CTAs that fill one (8 taps each)
 #define ISM_SHELL_BINS 8          // delay bins per CTA of the fused Chebyshev accumulation
 #define ISM_SD_BINS 32            // delay bins per CTA of the fused direct accumulation
 #define ISM_FILL_CTAS 304         // fused CTAs a launch set should have at least (two per SM of a GB300)
@@ -82,7 +87,7 @@ struct JobDev {
     int W_env;                // samples of the envelope fit window
     int vec4;                 // out rows 16-byte aligned (float4 stores allowed)
     float half_scale;         // FP16X2 records are scaled by this power of two
-    int use_cheb;             // FP32 accumulation through Chebyshev moments (32-tap window)
+    int use_cheb;             // FP32 accumulation through Chebyshev moments: the terms (0: not this form)
     int shell_groups;         // fused Chebyshev CTAs per RIR (ISM_SHELL_BINS bins each; 0 otherwise)
     int sparse;               // direct FP32 form, few images per bin: no sort, each image's taps added at once
     int adj_cheb;             // backward: fused Chebyshev adjoint (32-tap window; shell_groups CTAs per RIR)
@@ -116,7 +121,8 @@ struct JobDev {
     float* grad_rcv;          // [n_rcv][3]
     int gpart_base;           // first per-(RIR, bin) gradient record (x 12 floats); below 2^31
     int rgrad_base;           // first per-RIR gradient (float; 12 per RIR)
-    int lut_base;             // first entry (float) of the job's windowed-sinc table (LUT forms)
+    int lut_base;             // first entry (float) of the job's windowed-sinc table (LUT forms) or of the
+                              // Chebyshev coefficients of its tap functions (windows other than 32 taps)
     // diffuse tail
     float g2_lo;              // low part of g2 (g2 + g2_lo is the FP64 value to ~2^-48)
     int envelope;             // ISM_ENVELOPE_SABINE or ISM_ENVELOPE_LJ
@@ -157,7 +163,7 @@ struct WsPlan {
     size_t dtbl_off;       // float4 [tbl_total] (backward): dF/dbeta_lo, dF/dbeta_hi, d x_n / d x_s per axis index
     size_t rows_off;       // float  [rows_total]: per-bin window rows of the accumulation
     size_t amp_off;        // float  [rir_total]
-    size_t lut_off;        // float  [lut_total]: polyphase windowed-sinc tables (LUT form)
+    size_t lut_off;        // float  [lut_total]: polyphase windowed-sinc tables (LUT forms), Chebyshev coefficients
     size_t gpart_off;      // float  [gpart_total]: backward, per-(RIR, bin) gradients
     size_t rgrad_off;      // float  [rgrad_total]: backward, per-RIR gradients
     size_t env_off;        // float  [env_total]: per-job envelope tables (Lehmann-Johansson tails)
@@ -169,6 +175,7 @@ struct WsPlan {
     long long rows_total;
     long long rir_total;
     long long lut_total;
+    int cheb_tabs;         // tables of Chebyshev coefficients (one per window length other than 32 taps)
     long long gpart_total;
     long long rgrad_total;
     long long env_total;
