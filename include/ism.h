@@ -217,13 +217,15 @@ ism_status ism_workspace_status(const void* workspace, void* stream, uint32_t* f
  *   driver loads the library's device code and reserves the 64 MiB, so the
  *   first call on each device can block, and can fail (ISM_ERR_CUDA, e.g.
  *   out of memory); later calls cannot fail that way.  The first call whose
- *   simulation is large enough to run as two halves (see ism_set_lanes) also
- *   creates, once per host thread and device, two internal streams and three
- *   events.  A real-time caller should therefore make one warm-up call at
- *   set-up on each device and each host thread it will call from, outside
- *   its real-time path, and before any stream capture.
- *   Limit: a simulation needing more scratch than 64 MiB (ism_workspace_size)
- *   is rejected with ISM_ERR_UNSUPPORTED and nothing is launched.
+ *   simulation runs as two halves (see ism_set_lanes) also creates, once per
+ *   host thread and device, two internal streams and three events.  A
+ *   real-time caller should therefore make one warm-up call at set-up on each
+ *   device and each host thread it will call from, outside its real-time
+ *   path, and before any stream capture.
+ *   Limit: a simulation needing more scratch than 64 MiB -- what
+ *   ism_workspace_size reports, and for FP32 windows of other than 32 taps what
+ *   the form over binned image ids would take -- is rejected with
+ *   ISM_ERR_UNSUPPORTED and nothing is launched.
  *   Sharing: every call uses the same area and leaves its contents behind;
  *   the kernels reset what they need.  Two calls whose work overlaps on the
  *   GPU (different streams without ordering between them, or different host
@@ -572,10 +574,12 @@ typedef enum {
 } ism_stage;
 
 /* Internal concurrency (no counterpart in the paper; a deployment setting):
- * a forward call with enough work (about 2e7 image sources in reach) runs
- * as two halves, split by source, on two internal streams forked from and
- * joined back into the caller's stream, so that one half's enumeration
- * overlaps the other's accumulation.  n_lanes = 1 keeps every launch on the
+ * a forward call with enough work (about 2e7 image sources in reach) whose
+ * results are copied to the host (ism_simulate_host into pageable memory) or
+ * that is too large for one set of launches runs as two halves, split by
+ * source, on two internal streams forked from and joined back into the caller's
+ * stream, so that one half's copy overlaps the other's computation; a batch of
+ * more than 64 jobs alternates between them.  n_lanes = 1 keeps every launch on the
  * caller's stream (each kernel then runs alone, e.g. for timing it); 2 is
  * the default.  The results are bit-identical either way.  Process-wide. */
 ism_status ism_set_lanes(int n_lanes);

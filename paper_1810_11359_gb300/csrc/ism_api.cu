@@ -512,12 +512,16 @@ double images_in_reach(const Validated& v)
 }
 
 // Execution schedule of a forward call: launch sets (<= ISM_MAX_JOBS jobs
-// each) and the lane (internal stream) of each.  A call with enough work is
-// cut into two halves by source (or by receiver for one source) that run on
-// two lanes, so that one half's enumeration overlaps the other half's
-// accumulation; sets alternate between the lanes.  A sub-job keeps the
-// RIR index of its first RIR (the noise counter), so every RIR is computed
-// exactly as in the unsplit job.
+// each) and the lane (internal stream) of each; sets alternate between the
+// lanes.  A call with enough work whose results are copied to the host is cut
+// into two halves by source (or by receiver for one source), so that one half's
+// copy overlaps the other's computation; so is one that is too large for a
+// launch set.  Others run as one: the fused kernels leave the second half
+// nothing to overlap with, and halves have two last waves (a call, two halves
+// against one: 128 RIRs FP32 382 and 379 us, 64 RIRs FP16X2 629 and 566 us, 16
+// RIRs of 64 taps 352 and 320 us, 512 RIRs at 48 kHz 302 both).  A sub-job
+// keeps the RIR index of its first RIR (the noise counter), so every RIR is
+// computed exactly as in the unsplit job.
 struct Schedule {
     std::vector<std::vector<Validated>> sets;
     int lanes = 1;
@@ -525,12 +529,25 @@ struct Schedule {
 
 std::atomic<int> g_lanes{2};
 
-Schedule schedule(const std::vector<Validated>& vs)
+// Whether the jobs fit launch sets as they are.
+bool sets_fit(const std::vector<Validated>& vs, ism_precision prec)
+{
+    JobTable t;
+    WsPlan p;
+    for (size_t g = 0; g < vs.size(); g += ISM_MAX_JOBS)
+        if (plan(vs.data() + g, (int)std::min<size_t>(ISM_MAX_JOBS, vs.size() - g), prec, false, t, p) != ISM_OK) {
+            g_last_error.clear();
+            return false;
+        }
+    return true;
+}
+
+Schedule schedule(const std::vector<Validated>& vs, ism_precision prec, bool copies)
 {
     Schedule sc;
     double work = 0.0;
     for (const Validated& v : vs) work += images_in_reach(v) * (double)v.job.n_src * v.job.n_rcv;
-    const bool split = work >= 2.0e7 && g_lanes.load() >= 2;
+    const bool split = work >= 2.0e7 && g_lanes.load() >= 2 && (copies || !sets_fit(vs, prec));
     std::vector<Validated> halves[2];
     for (const Validated& v : vs) {
         const ism_job& j = v.job;
@@ -597,7 +614,7 @@ ism_status schedule_size(const Schedule& sc, ism_precision prec, size_t* bytes, 
 
 ism_status batch_size(const std::vector<Validated>& vs, ism_precision prec, size_t* bytes, bool backward = false)
 {
-    if (!backward) return schedule_size(schedule(vs), prec, bytes, nullptr);
+    if (!backward) return schedule_size(schedule(vs, prec, false), prec, bytes, nullptr);
     size_t best = 0;
     JobTable t;
     WsPlan p;
@@ -609,6 +626,16 @@ ism_status batch_size(const std::vector<Validated>& vs, ism_precision prec, size
     }
     *bytes = best;
     return ISM_OK;
+}
+
+// Simulation workspace of a host call, whichever way its results leave.
+ism_status host_size(const std::vector<Validated>& vs, ism_precision prec, size_t* bytes)
+{
+    size_t a = 0, b = 0;
+    ism_status s = schedule_size(schedule(vs, prec, false), prec, &a, nullptr);
+    if (s == ISM_OK) s = schedule_size(schedule(vs, prec, true), prec, &b, nullptr);
+    *bytes = std::max(a, b);
+    return s;
 }
 
 // The two internal streams (lanes) of the calling thread on the current
@@ -896,9 +923,9 @@ int copy_set_out(const std::vector<Validated>& set, const HostCopy* hc, cudaStre
 }
 
 ism_status run_batch(const std::vector<Validated>& vs, ism_precision prec, void* workspace, size_t ws_bytes,
-                     void* stream, const HostCopy* hc = nullptr)
+                     void* stream, const HostCopy* hc = nullptr, bool halves = false)
 {
-    const Schedule sc = schedule(vs);
+    const Schedule sc = schedule(vs, prec, hc != nullptr || halves);
     size_t need = 0, base1 = 0;
     ism_status s = schedule_size(sc, prec, &need, &base1);
     if (s != ISM_OK) return s;
@@ -1433,7 +1460,7 @@ ism_status ism_simulate_host(const ism_room* room, const float* pos_src, int n_s
     std::vector<Validated> vs;
     if ((s = validate_all(&j, 1, vs, false)) != ISM_OK) return s;
     size_t sim = 0;
-    if ((s = batch_size(vs, prec, &sim)) != ISM_OK) return s;
+    if ((s = host_size(vs, prec, &sim)) != ISM_OK) return s;
     // device layout: [simulation workspace | positions | output]
     size_t pos_off = align256(sim);
     size_t out_off = align256(pos_off + (size_t)(n_src + n_rcv) * 3 * sizeof(float));
@@ -1468,9 +1495,15 @@ ism_status ism_simulate_host(const ism_room* room, const float* pos_src, int n_s
 ism_status ism_host_workspace_size(const ism_room* room, int n_src, int n_rcv, const int nb_img[3], float Tmax,
                                    float fs, float Tdiff, float Tw, ism_precision prec, size_t* bytes)
 {
-    size_t sim = 0;
-    ism_status s = ism_workspace_size(room, n_src, n_rcv, nb_img, Tmax, fs, Tdiff, Tw, prec, &sim);
+    g_last_error.clear();
+    if (!room || !nb_img || !bytes) return fail(ISM_ERR_INVALID_ARG, "room, nb_img and bytes must not be NULL");
+    ism_status s = check_prec(prec);
     if (s != ISM_OK) return s;
+    ism_job j = make_job(room, nullptr, n_src, nullptr, n_rcv, nb_img, Tmax, fs, Tdiff, Tw, 0, nullptr);
+    std::vector<Validated> vs;
+    if ((s = validate_all(&j, 1, vs, false)) != ISM_OK) return s;
+    size_t sim = 0;
+    if ((s = host_size(vs, prec, &sim)) != ISM_OK) return s;
     int n_S = rir_len(Tmax, fs);
     size_t pos_off = align256(sim);
     size_t out_off = align256(pos_off + (size_t)(n_src + n_rcv) * 3 * sizeof(float));
@@ -1786,7 +1819,7 @@ extern "C" ism_status ism_simulate_noalloc(const ism_room* room, const float* po
     size_t need = 0;
     // (the limit counts the scratch of binned image ids, whichever kernels take the call: what
     // it admits does not change with them, and the fused forms need less)
-    if ((s = schedule_size(schedule(vs), prec, &need, nullptr, true)) != ISM_OK) return s;
+    if ((s = schedule_size(schedule(vs, prec, true), prec, &need, nullptr, true)) != ISM_OK) return s;
     if (need > ISM_NOALLOC_SCRATCH_BYTES)
         return fail(ISM_ERR_UNSUPPORTED,
                     "this simulation needs %zu bytes of scratch, above the %u bytes of the allocation-free "
@@ -1794,5 +1827,8 @@ extern "C" ism_status ism_simulate_noalloc(const ism_room* room, const float* po
                     need, (unsigned)ISM_NOALLOC_SCRATCH_BYTES);
     void* scratch = nullptr;
     if ((s = noalloc_scratch(&scratch)) != ISM_OK) return s;
-    return run_batch(vs, prec, scratch, ISM_NOALLOC_SCRATCH_BYTES, stream);
+    size_t whole = 0;   // (as one set of launches unless only halves fit)
+    const bool fits = schedule_size(schedule(vs, prec, false), prec, &whole, nullptr) == ISM_OK &&
+                      whole <= ISM_NOALLOC_SCRATCH_BYTES;
+    return run_batch(vs, prec, scratch, ISM_NOALLOC_SCRATCH_BYTES, stream, nullptr, !fits);
 }
