@@ -841,13 +841,8 @@ ism_status run_set(const std::vector<Validated>& set, ism_precision prec, size_t
         }
     void* stream = (void*)st;
     int e;
-    {
-        StageTimer tm(ISM_STAGE_GEOMETRY, st);
-        if ((e = ism_launch_geometry(t, p, ws, stream))) return cuda_fail(e, "geometry kernel");
-        tm.done(p.rir_total > 0);
-    }
     // envelope tables of Lehmann-Johansson tails (read by finalize and tail): on the side
-    // stream, joined back before finalize (on the launch stream while profiling, so that
+    // stream from the start, joined back before finalize (on the launch stream while profiling, so that
     // the stage times stay those of one stream)
     Side* side = nullptr;
     if (p.env_ctas > 0) {
@@ -862,6 +857,11 @@ ism_status run_set(const std::vector<Validated>& set, ism_precision prec, size_t
             if ((e = ism_launch_envelope(t, p, ws, stream))) return cuda_fail(e, "envelope kernel");
             tm.done(1);
         }
+    }
+    {
+        StageTimer tm(ISM_STAGE_GEOMETRY, st);
+        if ((e = ism_launch_geometry(t, p, ws, stream))) return cuda_fail(e, "geometry kernel");
+        tm.done(p.rir_total > 0);
     }
     {
         StageTimer tm(ISM_STAGE_ENUM_COUNT, st);

@@ -182,14 +182,19 @@ __global__ void __launch_bounds__(256) tail_kernel(const __grid_constant__ JobTa
 // (the average over one octant of directions u; log2 of the energy lost per
 // sample along u).  One CTA per job (envelope_nodes_kernel) builds the
 // Gauss-Legendre product rule (nodes by Newton's iteration on the Legendre
-// recurrence, FP64), the node rates g in float-float and the weights in FP32,
-// and E(t0); then four threads of envelope_kernel share each sample: each sums
-// a quarter of its n^2 terms 2^(-k g) with Kahan's compensated FP32 summation
-// (all terms positive: relative error ~2 ulp plus exp2f's 2 ulp), and the four
-// partial sums are added in FP64 in a fixed order (E(t0) likewise).  n =
+// recurrence, FP64), the node rates g in float-float, their ratios 2^-g and the
+// weights in FP32, and E(t0); then 16 threads of envelope_kernel share four
+// samples: each sums a sixteenth of their n^2 terms 2^(-k g) with Kahan's
+// compensated FP32 summation (all terms positive: relative error ~2 ulp plus
+// exp2f's 2 ulp and the ratio's, which differ from node to node), and the
+// partial sums are added in FP64 in a fixed order (E(t0) likewise).  Both
+// kernels are latency chains beside a narrow FP64 unit (one CTA per job, then
+// 64 samples per CTA): for 15 RIRs of 26,460 samples at 44.1 kHz 15 and 10 us,
+// 58 us together with five Newton steps of divisions, one thread's logarithms
+// and an exp2 per node and sample.  n =
 // clamp(ceil(K / 4) + 12, 16, 64) nodes per angle, K = (n_S / f_s) c
 // |(-ln rho_a / L_a)_a|, the largest exponent (in nepers) over the table.  A
-// job's node slot holds ISM_ENV_SLOT float4 {g hi, g lo, w, 0}, the last one
+// job's node slot holds ISM_ENV_SLOT float4 {g hi, g lo, w, 2^-g}, the last one
 // {n (int bits), 0, E(t0) as the two halves of an FP64}.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) envelope_nodes_kernel(const __grid_constant__ JobTable t,
@@ -201,58 +206,59 @@ __global__ void __launch_bounds__(256) envelope_nodes_kernel(const __grid_consta
     __shared__ double wg[ISM_ENV_MAX_NODES];
     __shared__ double sth[ISM_ENV_MAX_NODES], cth[ISM_ENV_MAX_NODES];
     __shared__ double gam[3];
-    __shared__ int n_s;
     __shared__ double part[256];
-    __shared__ double inv_m[ISM_ENV_MAX_NODES + 1];   // 1 / m for the Legendre recurrence
+    __shared__ double inv_d[ISM_ENV_MAX_NODES + 1];   // 1 / m for the Legendre recurrence
+    __shared__ float inv_m[ISM_ENV_MAX_NODES + 1];
     const double PI = 3.141592653589793238462643383279502884;
-    if (threadIdx.x == 0) {
-        double kn = 0.0;
-        for (int a = 0; a < 3; ++a) {
-            const double rho = fabs((double)ism_job_beta(J, 2 * a) * (double)ism_job_beta(J, 2 * a + 1));
-            const double nep = rho > 0.0 ? -log(rho) : 1.0e30;                 // nepers per reflection pair
-            gam[a] = rho > 0.0 ? nep / log(2.0) * (double)J.c / ((double)J.fs * J.L[a]) : 1.0e30;
-            const double ka = nep * (double)J.c * ((double)J.n_S / (double)J.fs) / J.L[a];
-            kn += ka * ka;
-        }
-        kn = sqrt(kn);
-        n_s = kn < 4.0 * (ISM_ENV_MAX_NODES - 12) ? max(16, (int)ceil(kn / 4.0) + 12) : ISM_ENV_MAX_NODES;
+    // GB300's FP64 unit is narrow and its chains long, so the FP64 work is spread over threads
+    // and kept to one evaluation of each function
+    __shared__ double nepers[3];
+    if ((int)threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        const double rho = fabs((double)ism_job_beta(J, 2 * a) * (double)ism_job_beta(J, 2 * a + 1));
+        const double per_m = rho > 0.0 ? -log2(rho) / J.L[a] : 1.0e30;   // log2 of the decay per metre along the axis
+        gam[a] = rho > 0.0 ? per_m * ((double)J.c / (double)J.fs) : 1.0e30;
+        nepers[a] = per_m * (0.69314718055994530942 * (double)J.c * ((double)J.n_S / (double)J.fs));
     }
-    if ((int)threadIdx.x <= ISM_ENV_MAX_NODES) inv_m[threadIdx.x] = threadIdx.x ? 1.0 / (double)threadIdx.x : 0.0;
+    if ((int)threadIdx.x >= 32 && (int)threadIdx.x <= 32 + ISM_ENV_MAX_NODES) {
+        const int m = (int)threadIdx.x - 32;
+        inv_d[m] = m ? 1.0 / (double)m : 0.0;
+        inv_m[m] = (float)inv_d[m];
+    }
     __syncthreads();
-    const int n = n_s;
+    const double kn = sqrt(nepers[0] * nepers[0] + nepers[1] * nepers[1] + nepers[2] * nepers[2]);
+    const int n = kn < 4.0 * (ISM_ENV_MAX_NODES - 12) ? max(16, (int)ceil(kn / 4.0) + 12) : ISM_ENV_MAX_NODES;
     // Gauss-Legendre nodes and weights on [-1, 1]: Newton on P_n from the asymptotic guess
     if ((int)threadIdx.x < n) {
         const int i = threadIdx.x;
-        // Newton from a guess within ~1e-3 of the root: three steps in FP32 (to ~1e-7), then
-        // two in FP64 (each doubles the correct digits); the weight takes the derivative of
-        // the last step (its point differs from the root by ~1e-16)
+        // Newton from a guess within ~1e-3 of the root: three steps in FP32 (to ~1e-7), then one
+        // in FP64 (to ~1e-14); the derivative at the new point, which the weight takes, from
+        // Legendre's equation, (1 - x^2) P'' = 2 x P' - n (n + 1) P
         float xf = cospif((i + 0.75f) / (n + 0.5f));
         for (int it = 0; it < 3; ++it) {
             float p0 = 1.0f, p1 = xf;
             for (int m = 2; m <= n; ++m) {
-                const float p2 = ((2.0f * m - 1.0f) * xf * p1 - (m - 1.0f) * p0) * (float)inv_m[m];
+                const float p2 = ((2.0f * m - 1.0f) * xf * p1 - (m - 1.0f) * p0) * inv_m[m];
                 p0 = p1;
                 p1 = p2;
             }
             const float dpf = n * (xf * p1 - p0) / (xf * xf - 1.0f);
             xf -= p1 / dpf;
         }
-        double x = (double)xf;
-        double dp = 1.0;
-        for (int it = 0; it < 2; ++it) {
-            double p0 = 1.0, p1 = x;
-            for (int m = 2; m <= n; ++m) {
-                const double p2 = ((2.0 * m - 1.0) * x * p1 - (m - 1.0) * p0) * inv_m[m];
-                p0 = p1;
-                p1 = p2;
-            }
-            dp = n * (x * p1 - p0) / (x * x - 1.0);
-            x -= p1 / dp;
+        const double x0 = (double)xf;
+        double p0 = 1.0, p1 = x0;
+        for (int m = 2; m <= n; ++m) {   // P_m = (2 - 1/m) x P_(m-1) - (1 - 1/m) P_(m-2): one dependent FMA a step
+            const double p2 = fma((2.0 - inv_d[m]) * x0, p1, -(1.0 - inv_d[m]) * p0);
+            p0 = p1;
+            p1 = p2;
         }
-        wg[i] = 2.0 / ((1.0 - x * x) * dp * dp);
-        const double ang = (x + 1.0) * (PI / 4.0);   // [-1, 1] -> [0, pi/2]
-        sth[i] = sin(ang);
-        cth[i] = cos(ang);
+        const double om = 1.0 / (1.0 - x0 * x0);
+        const double dp = n * (p0 - x0 * p1) * om;
+        const double dx = -p1 / dp;
+        const double dp1 = dp + dx * (2.0 * x0 * dp - (double)(n * (n + 1)) * p1) * om;
+        const double x = x0 + dx;
+        wg[i] = 2.0 / ((1.0 - x * x) * dp1 * dp1);
+        sincospi(0.25 * (x + 1.0), &sth[i], &cth[i]);   // the angle, [-1, 1] -> [0, pi/2]
     }
     __syncthreads();
     // nodes (theta_i, phi_j): u = (sin t cos p, sin t sin p, cos t), weight (pi/4)^2 w_i w_j sin t (2 / pi);
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(256) envelope_nodes_kernel(const __grid_consta
         const float hi = (float)gr;
         const float lo = gr < 1.0e29 ? (float)(gr - (double)hi) : 0.0f;
         const float w = (float)(wg[i] * wg[j] * sth[i] * (PI / 8.0));
-        slot[e] = make_float4(hi, lo, w, 0.0f);
+        slot[e] = make_float4(hi, lo, w, ism_exp2_neg(ff{hi, lo}, 1));
         const float y = __fsub_rn(__fmul_rn(w, ism_exp2_neg(ff{hi, lo}, J.n_ism)), comp);
         const float tt = __fadd_rn(s, y);
         comp = __fsub_rn(__fsub_rn(tt, s), y);
@@ -289,14 +295,15 @@ __global__ void __launch_bounds__(4 * ISM_ENV_CHUNK) envelope_kernel(const __gri
                                                                  const float4* __restrict__ nodes,
                                                                  float* __restrict__ env)
 {
+    constexpr int PARTS = 16;   // threads that share four samples
     extern __shared__ __align__(16) unsigned char smem[];
     const long long g = blockIdx.x;
     const int jid = ism_find_job(t, g, [](const JobDev& j) { return (long long)j.env_cta_base; });
     const JobDev& J = t.j[jid];
     const int chunk = (int)(g - J.env_cta_base);
     const float4* slot = nodes + (long long)J.env_slot * ISM_ENV_SLOT;
-    float4* nd = reinterpret_cast<float4*>(smem);   // [n * n] {g hi, g lo, w, 0}
-    __shared__ float part[4][ISM_ENV_CHUNK];
+    float4* nd = reinterpret_cast<float4*>(smem);   // [n * n] {g hi, g lo, w, 2^-g}
+    __shared__ float part[PARTS][ISM_ENV_CHUNK];
     const float4 head = slot[ISM_ENV_SLOT - 1];
     const int n = __float_as_int(head.x);
     const double E0 = __longlong_as_double((long long)(((unsigned long long)__float_as_uint(head.w) << 32) |
@@ -304,28 +311,38 @@ __global__ void __launch_bounds__(4 * ISM_ENV_CHUNK) envelope_kernel(const __gri
     const int nn = n * n;
     for (int e = threadIdx.x; e < nn; e += blockDim.x) nd[e] = slot[e];
     __syncthreads();
-    // sample ks of the chunk, quarter qp of the nodes (i = qp, qp + 4, ...)
-    const int ks = (int)threadIdx.x % ISM_ENV_CHUNK, qp = (int)threadIdx.x / ISM_ENV_CHUNK;
+    // samples k .. k + 3 of the chunk, part qp of the nodes (i = qp, qp + 16, ...): one exp2 a
+    // node for the first sample, the others by the node's ratio 2^-g
+    const int qp = (int)threadIdx.x % PARTS, ks = 4 * ((int)threadIdx.x / PARTS);
     const int k = J.env_k0 + chunk * ISM_ENV_CHUNK + ks;
-    float s = 0.0f, comp = 0.0f;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, comp[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (k < J.n_S && E0 > 0.0) {
-        for (int i = qp; i < nn; i += 4) {
+        for (int i = qp; i < nn; i += PARTS) {
             const float4 q = nd[i];
-            const float y = __fsub_rn(__fmul_rn(q.z, ism_exp2_neg(ff{q.x, q.y}, k)), comp);
-            const float tt = __fadd_rn(s, y);
-            comp = __fsub_rn(__fsub_rn(tt, s), y);
-            s = tt;
+            float v = __fmul_rn(q.z, ism_exp2_neg(ff{q.x, q.y}, k));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float y = __fsub_rn(v, comp[u]);
+                const float tt = __fadd_rn(s[u], y);
+                comp[u] = __fsub_rn(__fsub_rn(tt, s[u]), y);
+                s[u] = tt;
+                v = __fmul_rn(v, q.w);
+            }
         }
     }
-    part[qp][ks] = s;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) part[qp][ks + u] = s[u];
     __syncthreads();
-    if (qp != 0 || k >= J.n_S) return;
+    const int e = threadIdx.x;
+    const int ke = J.env_k0 + chunk * ISM_ENV_CHUNK + e;
+    if (e >= ISM_ENV_CHUNK || ke >= J.n_S) return;
     float v = 0.0f;
     if (E0 > 0.0) {
-        const double E = (((double)part[0][ks] + part[1][ks]) + part[2][ks]) + part[3][ks];
+        double E = 0.0;
+        for (int p = 0; p < PARTS; ++p) E += (double)part[p][e];
         v = (float)sqrt(E / E0);
     }
-    env[J.env_base + (k - J.env_k0)] = v;
+    env[J.env_base + (ke - J.env_k0)] = v;
 }
 
 __global__ void noise_kernel(uint64_t seed, uint32_t rir, uint32_t k0, int n, float* z)
