@@ -177,6 +177,9 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
     long long set_cols = 0;   // grid columns x RIRs over the launch set
     for (int i = 0; i < n; ++i)
         set_cols += (long long)vs[i].job.nb_img[0] * vs[i].job.nb_img[1] * vs[i].job.n_src * vs[i].job.n_rcv;
+    long long fin_set = 0;    // finalize CTAs of 2048 samples over the launch set
+    for (int i = 0; i < n; ++i) fin_set += (long long)vs[i].job.n_src * vs[i].job.n_rcv * ((vs[i].n_ism + 2047) / 2048);
+    const bool fin_small = fin_set < ISM_FILL_CTAS;
     long long rir = 0, hist = 0, tbl = 0, ecta = 0, acta = 0, adta = 0, tcta = 0, fcta = 0, rows = 0, ids = 0, lut = 0,
               gpart = 0, srir = 0, scta = 0, env = 0, vcta = 0, sdc = 0, vslot = 0, sdrir = 0;
     int sd_gmax = 0;   // most shells of a fused direct RIR
@@ -269,7 +272,8 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
         J.adj_cta_base = adta;
         J.tail_cta_base = tcta;
         J.fin_cta_base = fcta;
-        J.fin_chunk = std::max(2048, (J.W_env + 255) / 256 * 256);
+        // (shorter chunks where a launch has few: finalize waits for memory, not for arithmetic)
+        J.fin_chunk = std::max(fin_small ? 1024 : 2048, (J.W_env + 255) / 256 * 256);
         J.fin_chunks = std::max(1, (v.n_ism + J.fin_chunk - 1) / J.fin_chunk);
         J.rows_base = rows;
         J.lut_base = lut;
