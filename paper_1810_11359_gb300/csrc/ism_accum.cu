@@ -3,13 +3,13 @@
 #include "ism_accum.cuh"
 
 int ism_launch_accum(const JobTable& t, const WsPlan& p, char* ws, ism_precision prec, void* stream,
-                     int* launched)
+                     void* direct_stream, int* launched)
 {
     // the fused kernels (32-tap windows: Chebyshev moments or every tap evaluated), then
     // the per-tap kernel over binned ids for the other windows
     int a = 0, b = 0, c = 0;
-    int rc = ism_launch_accum_cheb(t, p, ws, stream, &a);
-    if (!rc) rc = ism_launch_accum_shell_direct(t, p, ws, prec, stream, &b);
+    int rc = ism_launch_accum_shell_direct(t, p, ws, prec, direct_stream, &b);
+    if (!rc) rc = ism_launch_accum_cheb(t, p, ws, stream, &a);
     if (!rc) {
         switch (prec) {
         case ISM_PREC_FP32:

@@ -733,12 +733,16 @@ bool profiling_on()
 }
 
 // Side stream of the calling thread on the current device, with the events that fork
-// it from and join it back into a launch stream (the envelope kernels run there,
-// beside the enumeration and the accumulation they do not depend on).
+// it from (at the start of a launch set, and after its geometry) and join it back
+// into a launch stream.  What does not depend on the launch stream's next kernels runs
+// there: the envelope kernels, and in batches that hold both dense and sparse rooms
+// the fused direct kernel beside the Chebyshev one (either leaves SMs idle at its end,
+// and the direct one's few long CTAs do not fill the GPU: 32 rooms of a service, 282
+// RIRs, 138 -> 120 us a call).
 struct Side {
     int dev = -1;
     cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaEvent_t fork = nullptr, fork2 = nullptr, join = nullptr;
 };
 
 int side_of_device(Side** out)
@@ -752,6 +756,7 @@ int side_of_device(Side** out)
     if (S.dev != d) {
         if ((e = (int)cudaStreamCreateWithFlags(&S.s, cudaStreamNonBlocking))) return e;
         if ((e = (int)cudaEventCreateWithFlags(&S.fork, cudaEventDisableTiming))) return e;
+        if ((e = (int)cudaEventCreateWithFlags(&S.fork2, cudaEventDisableTiming))) return e;
         if ((e = (int)cudaEventCreateWithFlags(&S.join, cudaEventDisableTiming))) return e;
         S.dev = d;
     }
@@ -845,22 +850,21 @@ ism_status run_set(const std::vector<Validated>& set, ism_precision prec, size_t
         }
     void* stream = (void*)st;
     int e;
-    // envelope tables of Lehmann-Johansson tails (read by finalize and tail): on the side
-    // stream from the start, joined back before finalize (on the launch stream while profiling, so that
-    // the stage times stay those of one stream)
+    // (everything on the launch stream while profiling, so that the stage times stay those of
+    // one stream)
+    const bool mixed = t.any_cheb && p.shell_ctas > 0 && p.sd_ctas > 0;
     Side* side = nullptr;
-    if (p.env_ctas > 0) {
-        if (!profiling_on()) {
-            if ((e = side_of_device(&side))) return cuda_fail(e, "internal stream");
-            if ((e = (int)cudaEventRecord(side->fork, st))) return cuda_fail(e, "event record");
-            if ((e = (int)cudaStreamWaitEvent(side->s, side->fork, 0))) return cuda_fail(e, "stream wait");
-            if ((e = ism_launch_envelope(t, p, ws, (void*)side->s))) return cuda_fail(e, "envelope kernel");
-            if ((e = (int)cudaEventRecord(side->join, side->s))) return cuda_fail(e, "event record");
-        } else {
-            StageTimer tm(ISM_STAGE_TAIL, st);
-            if ((e = ism_launch_envelope(t, p, ws, stream))) return cuda_fail(e, "envelope kernel");
-            tm.done(1);
-        }
+    if ((p.env_ctas > 0 || mixed) && !profiling_on() && (e = side_of_device(&side)))
+        return cuda_fail(e, "internal stream");
+    // envelope tables of Lehmann-Johansson tails (read by finalize and tail)
+    if (p.env_ctas > 0 && side) {
+        if ((e = (int)cudaEventRecord(side->fork, st))) return cuda_fail(e, "event record");
+        if ((e = (int)cudaStreamWaitEvent(side->s, side->fork, 0))) return cuda_fail(e, "stream wait");
+        if ((e = ism_launch_envelope(t, p, ws, (void*)side->s))) return cuda_fail(e, "envelope kernel");
+    } else if (p.env_ctas > 0) {
+        StageTimer tm(ISM_STAGE_TAIL, st);
+        if ((e = ism_launch_envelope(t, p, ws, stream))) return cuda_fail(e, "envelope kernel");
+        tm.done(1);
     }
     {
         StageTimer tm(ISM_STAGE_GEOMETRY, st);
@@ -890,10 +894,20 @@ ism_status run_set(const std::vector<Validated>& set, ism_precision prec, size_t
             ++launched;
         }
         int acc_launched = 0;
-        if ((e = ism_launch_accum(t, p, ws, prec, stream, &acc_launched))) return cuda_fail(e, "accumulation kernel");
+        void* direct = stream;
+        if (mixed && side) {
+            if ((e = (int)cudaEventRecord(side->fork2, st))) return cuda_fail(e, "event record");
+            if ((e = (int)cudaStreamWaitEvent(side->s, side->fork2, 0))) return cuda_fail(e, "stream wait");
+            direct = (void*)side->s;
+        }
+        if ((e = ism_launch_accum(t, p, ws, prec, stream, direct, &acc_launched)))
+            return cuda_fail(e, "accumulation kernel");
         tm.done(launched + acc_launched);
     }
-    if (side && (e = (int)cudaStreamWaitEvent(st, side->join, 0))) return cuda_fail(e, "stream wait");
+    if (side) {
+        if ((e = (int)cudaEventRecord(side->join, side->s))) return cuda_fail(e, "event record");
+        if ((e = (int)cudaStreamWaitEvent(st, side->join, 0))) return cuda_fail(e, "stream wait");
+    }
     {
         StageTimer tm(ISM_STAGE_FINALIZE, st);
         if ((e = ism_launch_finalize(t, p, ws, stream))) return cuda_fail(e, "finalize kernel");

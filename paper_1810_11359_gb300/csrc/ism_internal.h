@@ -231,7 +231,7 @@ int ism_launch_geometry(const JobTable& t, const WsPlan& p, char* ws, void* stre
 int ism_launch_enum(const JobTable& t, const WsPlan& p, char* ws, bool scatter, void* stream);
 int ism_launch_scan(const WsPlan& p, char* ws, void* stream);
 int ism_launch_accum(const JobTable& t, const WsPlan& p, char* ws, ism_precision prec, void* stream,
-                     int* launched);
+                     void* direct_stream, int* launched);   // (the fused direct form on direct_stream)
 int ism_launch_accum_fp16(const JobTable& t, const WsPlan& p, char* ws, void* stream, int* launched);
 int ism_launch_accum_bf16(const JobTable& t, const WsPlan& p, char* ws, void* stream, int* launched);
 int ism_launch_accum_lut(const JobTable& t, const WsPlan& p, char* ws, void* stream, int* launched);
