@@ -9,6 +9,7 @@ raise.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import threading
 from typing import Optional, Sequence
@@ -60,6 +61,10 @@ class ism_job(ctypes.Structure):
 class ism_grad_job(ctypes.Structure):
     _fields_ = [("job", ism_job), ("grad_out", ctypes.c_void_p), ("grad_beta", ctypes.c_void_p),
                 ("grad_src", ctypes.c_void_p), ("grad_rcv", ctypes.c_void_p)]
+
+
+# numpy's view of the two (its conversion of a ctypes struct takes ~50 us, hence once)
+_JOB_DTYPE, _GRAD_JOB_DTYPE = np.dtype(ism_job), np.dtype(ism_grad_job)
 
 
 class ism_server_config(ctypes.Structure):
@@ -312,6 +317,16 @@ def _workspace(ws, nbytes):
     return ws.get(nbytes)
 
 
+def _positions(x, dev):
+    """[n, 3] contiguous FP32 tensor on dev (x itself where it is one already: the general
+    conversion takes ~10 us)."""
+    torch = _torch()
+    if (isinstance(x, torch.Tensor) and x.dtype == torch.float32 and x.device == dev and x.dim() == 2
+            and x.shape[1] == 3 and x.is_contiguous()):
+        return x
+    return torch.as_tensor(x, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
+
+
 def ism_simulate(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, Tdiff=0.0, Tw=0.0, c=343.0, prec: str = "fp32",
                  seed: int = 0, out=None, workspace: Optional[Workspace] = None, stream=None,
                  mic_pattern: str = "omni", orient_rcv=None, envelope: str = "sabine"):
@@ -323,8 +338,8 @@ def ism_simulate(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, Tdiff=0.0, Tw=0.0,
     envelope: power envelope of the diffuse tail (an ENVELOPES name)."""
     torch = _torch()
     dev = torch.device("cuda", torch.cuda.current_device())
-    ps = torch.as_tensor(pos_src, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
-    pr = torch.as_tensor(pos_rcv, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
+    ps = _positions(pos_src, dev)
+    pr = _positions(pos_rcv, dev)
     if out is None:
         out = torch.empty((ps.shape[0], pr.shape[0], _rir_len(Tmax, fs)), dtype=torch.float32, device=dev)
     if mic_pattern != "omni" or envelope != "sabine":   # these travel in the job struct: the batch entry point
@@ -406,8 +421,8 @@ def ism_simulate_noalloc(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, Tdiff=0.0,
     Calls must not overlap on the GPU; see include/ism.h."""
     torch = _torch()
     dev = torch.device("cuda", torch.cuda.current_device())
-    ps = torch.as_tensor(pos_src, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
-    pr = torch.as_tensor(pos_rcv, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
+    ps = _positions(pos_src, dev)
+    pr = _positions(pos_rcv, dev)
     n_S = ism_rir_length(Tmax, fs)
     if out is None:
         out = torch.empty((ps.shape[0], pr.shape[0], n_S), dtype=torch.float32, device=dev)
@@ -451,6 +466,15 @@ def make_job(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, out, Tdiff=0.0, Tw=0.0
     return j
 
 
+def _row_bytes(t) -> int:
+    """Bytes of one entry of the first axis of a contiguous FP32 tensor."""
+    return 4 * math.prod(t.shape[1:])
+
+
+def _addresses(base: int, step: int, n: int) -> np.ndarray:
+    return np.arange(n, dtype=np.uint64) * np.uint64(step) + np.uint64(base)
+
+
 def make_jobs_strided(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, out, Tdiff=0.0, Tw=0.0, c=343.0, seed=0):
     """B jobs over batched CUDA tensors pos_src [B, S, 3], pos_rcv [B, M, 3],
     out [B, S, M, n_S] (contiguous FP32; they must stay alive during the call):
@@ -461,22 +485,21 @@ def make_jobs_strided(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, out, Tdiff=0.
     B = int(pos_src.shape[0])
     S, M = int(pos_src.shape[1]), int(pos_rcv.shape[1])
     arr = (ism_job * B)()
-    v = np.frombuffer(arr, dtype=np.dtype(ism_job), count=B)
+    v = np.frombuffer(arr, dtype=_JOB_DTYPE, count=B)
+    j = ism_job()   # what the jobs share, copied to all of them at once
+    j.room.c, j.n_src, j.n_rcv = float(c), S, M
+    j.Tmax, j.fs, j.Tdiff, j.Tw = float(Tmax), float(fs), float(Tdiff or 0.0), float(Tw or 0.0)
+    j.seed = int(seed) & (2 ** 64 - 1)
+    v[:] = np.frombuffer(j, dtype=_JOB_DTYPE, count=1)
     v["room"]["L"] = np.asarray(L, np.float64).reshape(B, 3)
+    v["nb_img"] = np.asarray(nb_img, np.int32).reshape(B, 3)
     if hasattr(beta, "data_ptr"):
-        v["beta_dev"] = np.uint64(beta.data_ptr()) + np.arange(B, dtype=np.uint64) * np.uint64(24)
+        v["beta_dev"] = _addresses(beta.data_ptr(), 24, B)
     else:
         v["room"]["beta"] = np.asarray(beta, np.float64).reshape(B, 6).astype(np.float32)
-    v["room"]["c"] = np.float32(c)
-    idx = np.arange(B, dtype=np.uint64)
-    v["pos_src"] = np.uint64(pos_src.data_ptr()) + idx * np.uint64(S * 3 * 4)
-    v["n_src"] = S
-    v["pos_rcv"] = np.uint64(pos_rcv.data_ptr()) + idx * np.uint64(M * 3 * 4)
-    v["n_rcv"] = M
-    v["nb_img"] = np.asarray(nb_img, np.int32).reshape(B, 3)
-    v["Tmax"], v["fs"], v["Tdiff"], v["Tw"] = float(Tmax), float(fs), float(Tdiff or 0.0), float(Tw or 0.0)
-    v["seed"] = int(seed) & (2 ** 64 - 1)
-    v["out"] = np.uint64(out.data_ptr()) + idx * np.uint64(out[0].numel() * 4)
+    v["pos_src"] = _addresses(pos_src.data_ptr(), S * 3 * 4, B)
+    v["pos_rcv"] = _addresses(pos_rcv.data_ptr(), M * 3 * 4, B)
+    v["out"] = _addresses(out.data_ptr(), _row_bytes(out), B)
     return arr
 
 
@@ -486,11 +509,10 @@ def make_grad_jobs_strided(jobs, grad_out, grad_beta, grad_src, grad_rcv):
     grad_rcv [B, M, 3] (the jobs' out is not touched; it is set to grad_out)."""
     B = len(jobs)
     arr = (ism_grad_job * B)()
-    v = np.frombuffer(arr, dtype=np.dtype(ism_grad_job), count=B)
-    v["job"] = np.frombuffer(jobs, dtype=np.dtype(ism_job), count=B)
-    idx = np.arange(B, dtype=np.uint64)
+    v = np.frombuffer(arr, dtype=_GRAD_JOB_DTYPE, count=B)
+    v["job"] = np.frombuffer(jobs, dtype=_JOB_DTYPE, count=B)
     for name, t in (("grad_out", grad_out), ("grad_beta", grad_beta), ("grad_src", grad_src), ("grad_rcv", grad_rcv)):
-        v[name] = np.uint64(t.data_ptr()) + idx * np.uint64(t[0].numel() * 4)
+        v[name] = _addresses(t.data_ptr(), _row_bytes(t), B)
     v["job"]["out"] = v["grad_out"]
     return arr
 
@@ -548,8 +570,8 @@ def ism_simulate_backward(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, grad_out,
     dLoss/dh = grad_out [n_src, n_rcv, n_S] through the image-source samples."""
     torch = _torch()
     dev = torch.device("cuda", torch.cuda.current_device())
-    ps = torch.as_tensor(pos_src, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
-    pr = torch.as_tensor(pos_rcv, dtype=torch.float32).to(dev).reshape(-1, 3).contiguous()
+    ps = _positions(pos_src, dev)
+    pr = _positions(pos_rcv, dev)
     go = torch.as_tensor(grad_out, dtype=torch.float32).to(dev).contiguous()
     gb = torch.empty(6, dtype=torch.float32, device=dev)
     gs = torch.empty((ps.shape[0], 3), dtype=torch.float32, device=dev)
@@ -706,7 +728,7 @@ class Server:
         if n == 0:
             return []
         arr = (ism_job * n)()
-        v = np.frombuffer(arr, dtype=np.dtype(ism_job), count=n)
+        v = np.frombuffer(arr, dtype=_JOB_DTYPE, count=n)
         v["room"]["L"] = np.array([r["L"] for r in reqs], np.float64).reshape(n, 3)
         v["room"]["beta"] = np.array([r["beta"] for r in reqs], np.float64).reshape(n, 6).astype(np.float32)
         v["room"]["c"] = [float(r.get("c", 343.0)) for r in reqs]

@@ -110,4 +110,4 @@ def rir(L, beta, pos_src, pos_rcv, Tmax: float, fs: float, Tw: float = 0.0, nb_i
     spec = _Spec(L=Lh, nb_img=nb, Tmax=float(Tmax), fs=float(fs), Tdiff=float(Tdiff or 0.0), Tw=float(Tw or 0.0),
                  c=float(c), seed=int(seed), prec=prec, workspace=workspace)
     out = _RoomsRIR.apply(beta_t, ps, pr, spec)
-    return out[0] if single else out
+    return out.view(out.shape[1:]) if single else out   # (a view: out[0] would copy its gradient)
