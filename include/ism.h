@@ -498,19 +498,20 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
 
 /* The same filtering with a choice of method and a caller-owned workspace.
  * The paper filters with batched FFTs and overlap-add; ISM_AURALIZE_FFT does
- * it in the frequency domain with FFTs written for this library (FP32,
- * four-step: length-N DFTs, N the power of two >= n_x + n_S - 1, at most 2^20, split
- * as N = R C into shared-memory DFTs of R and C points).  Two microphones
- * share one complex sequence (real and imaginary parts), the segment
- * spectra X_p times the pair spectra are summed over the points in ascending
- * order (the overlap-add, in the frequency domain), and one inverse DFT per
- * pair gives both outputs; results are identical run to run.  Its error is
+ * it in the frequency domain with FFTs written for this library, FP32, in one
+ * of two forms by their operation counts: overlap-save with 4096-point DFTs
+ * (many short segments), or four-step (length-N DFTs, N the power of two >=
+ * n_x + n_S - 1, at most 2^20, split as N = R C into shared-memory DFTs of R
+ * and C points).  Two microphones share one complex sequence (real and
+ * imaginary parts), the segment spectra X_p times the pair spectra are summed
+ * over the points in a fixed order (the overlap-add, in the frequency
+ * domain), and one inverse DFT per pair (and block) gives both outputs;
+ * results are identical run to run.  Its error is
  * that of an FP32 FFT: a few 1e-7 of the largest sum |x| * |h|, spread over
  * all outputs.  ISM_AURALIZE_DIRECT is ism_auralize (no workspace).
- * ISM_AURALIZE_AUTO takes the FFT form when its operation count is less than
- * 1 / 2.55 of the direct form's (n_mics n_x n_S multiply-adds; the ratio of the
- * two forms' measured rates on GB300) and the workspace holds at least one
- * chunk, else the direct form.
+ * ISM_AURALIZE_AUTO takes the FFT form when it is estimated to be faster than
+ * the direct form (n_mics n_x n_S multiply-adds; rates measured on GB300) and
+ * the workspace holds at least one chunk, else the direct form.
  *   workspace  device, 256-byte aligned, >= ism_auralize_workspace_size()
  *              bytes for the FFT form (scratch; may be NULL for DIRECT);
  *              a larger workspace processes more points per chunk.

@@ -1584,13 +1584,12 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
     return ISM_OK;
 }
 
-// Operation counts deciding the automatic choice of ism_auralize_ex: the
-// direct form does n_mics n_x n_S multiply-adds; the FFT form about 4 N log2 N
-// lane operations per length-N DFT (one per segment, one per microphone pair
-// and point, one inverse per pair) and 4 per product of spectra.  Measured on
-// the 48 kHz array's filtering, the direct form runs 2.55 times as many of its
-// units per second as the FFT form of its own (20.5 T multiply-adds/s against
-// 8.0 T operations/s), so the FFT form is taken above that ratio.
+// The automatic choice of ism_auralize_ex, from times estimated at measured rates: the
+// direct form does n_mics n_x n_S multiply-adds (20.5 T/s on the 48 kHz array's
+// filtering); the four-step FFT form about 4 N log2 N lane operations per length-N DFT
+// (one per segment, one per microphone pair and point, one inverse per pair) and 4 per
+// product of spectra (8.0 T/s); the overlap-save form as its estimate says.  64 points x
+// 2 microphones, RIRs of 4800 samples: 129 us direct, 33 us overlap-save.
 static bool auralize_fft_pays(int n_x, int n_points, int n_mics, int n_S)
 {
     const long long n_out = (long long)n_x + n_S - 1;
@@ -1601,7 +1600,7 @@ static bool auralize_fft_pays(int n_x, int n_points, int n_mics, int n_S)
     const double pairs = (double)((n_mics + 1) / 2);
     const double fft = ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * logN + (double)n_points * pairs * 4.0 * N;
     const double direct = (double)n_mics * (double)n_x * (double)n_S;
-    return direct > 2.55 * fft;
+    return direct > 2.55 * fft || direct / 2.05e13 > ism_auralize_ols_seconds(n_x, n_points, n_mics, n_S);
 }
 
 static ism_status auralize_args(const float* signal, int n_x, const float* rirs, int n_points, int n_mics, int n_S,
@@ -1660,7 +1659,14 @@ ism_status ism_auralize_ex(const float* signal, int n_x, const float* rirs, int 
                         (long long)n_x + n_S - 1);
         if (r == -2)
             return fail(ISM_ERR_WORKSPACE_TOO_SMALL, "workspace of %zu bytes holds no chunk of the FFT form", ws_bytes);
-        int e = ism_launch_auralize_fft(signal, rirs, starts, out, pl, static_cast<char*>(workspace), stream);
+        // many short segments: overlap-save with one short DFT length (its choice does not
+        // depend on the workspace's size, nor then the result)
+        AoPlan ol;
+        const size_t seq = (size_t)pl.N * 8;   // one point's chunk and the spectra: the least workspace
+        const size_t least = (size_t)(1 + pl.n_grp) * pl.n_pairs * seq + (size_t)(1 + pl.n_pairs) * seq;
+        int e = ism_auralize_ols_plan(n_x, n_points, n_mics, n_S, starts == nullptr, pl.logN, least, &ol)
+                    ? ism_launch_auralize_ols(signal, rirs, starts, out, ol, static_cast<char*>(workspace), stream)
+                    : ism_launch_auralize_fft(signal, rirs, starts, out, pl, static_cast<char*>(workspace), stream);
         if (e) return cuda_fail(e, "auralization (FFT) kernels");
         return ISM_OK;
     }

@@ -222,6 +222,17 @@ struct AfPlan {
     int n_grp;          // point groups of the row pass (partial spectra summed in group order)
 };
 
+// Plan of the overlap-save form of the moving-source filtering (ism_auralize_ols.cu).
+struct AoPlan {
+    int n_x, P, M, n_S, n_out, n_pairs;
+    int Lb;      // samples of a piece of a segment, at most
+    int V;       // outputs per block: 4096 - Lb + 1
+    int NB;      // blocks
+    int slots;   // pieces, with gaps
+    int G;       // groups of pieces per block (their sums are added in group order)
+    size_t desc_off, t1_off, x_off, y_off;   // in the workspace
+};
+
 // Sets the calling thread's ism_last_error_message() and returns s.
 ism_status ism_fail_message(ism_status s, const char* fmt, ...);
 
@@ -250,6 +261,11 @@ int ism_launch_auralize(const float* x, int n_x, const float* h, int n_points, i
                         float* y, void* stream);
 int ism_auralize_fft_plan(int n_x, int n_points, int n_mics, int n_S, size_t ws_bytes, AfPlan* out, size_t* need);
 int ism_launch_auralize_fft(const float* x, const float* h, const int* starts, float* y, const AfPlan& pl, char* ws,
+                            void* stream);
+double ism_auralize_ols_seconds(int n_x, int n_points, int n_mics, int n_S);
+bool ism_auralize_ols_plan(int n_x, int n_points, int n_mics, int n_S, bool uniform, int logN, size_t ws_min,
+                           AoPlan* out);
+int ism_launch_auralize_ols(const float* x, const float* h, const int* starts, float* y, const AoPlan& pl, char* ws,
                             void* stream);
 int ism_launch_beta_sabine(const double* L, const double* T60, const double* w, int negative, int n,
                            double* beta_out, int* status, void* stream);
