@@ -1600,7 +1600,7 @@ static bool auralize_fft_pays(int n_x, int n_points, int n_mics, int n_S)
     const double pairs = (double)((n_mics + 1) / 2);
     const double fft = ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * logN + (double)n_points * pairs * 4.0 * N;
     const double direct = (double)n_mics * (double)n_x * (double)n_S;
-    return direct > 2.55 * fft || direct / 2.05e13 > ism_auralize_ols_seconds(n_x, n_points, n_mics, n_S);
+    return direct > 2.55 * fft || 1.0e-5 + direct / 2.05e13 > ism_auralize_ols_seconds(n_x, n_points, n_mics, n_S);
 }
 
 static ism_status auralize_args(const float* signal, int n_x, const float* rirs, int n_points, int n_mics, int n_S,

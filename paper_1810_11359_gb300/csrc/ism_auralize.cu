@@ -6,12 +6,16 @@
 // on the FMA pipe (the RIRs are long, the signal is short, and the sum has a
 // fixed order).
 //
-// One CTA owns 128 consecutive output samples and up to 8 microphones; its 4
-// warps split the segments that reach the tile round-robin and add their
-// partial sums in warp order at the end.  Lane l of a warp owns the outputs
-// T0 + 4 l + r, r = 0 .. 3, for the 8 microphones (32 accumulators).  For one
-// segment the taps k that connect it to the tile are walked in chunks of 128:
-// the chunk's taps of the 8 microphones and the signal window it needs (the
+// One CTA owns 128 consecutive output samples and up to 8 microphones (1, 2, 4 or
+// 8, the least that holds the call's).  Lane l of a warp owns the outputs
+// T0 + 4 l + r, r = 0 .. 3, for the microphones (32 accumulators for 8).  For one
+// segment the taps k that connect it to the tile are walked in chunks of 128;
+// the chunks of all segments are dealt to the CTA's 16 warps in turn, which add
+// their partial sums in warp order at the end.  (16 points x 1 microphone, RIRs
+// of 9600 samples, a signal of 57,600: 337 us with 8 microphones' sums always
+// and whole segments dealt to 4 warps, 49 us now; 30 x 5, 16,000, 48,000: 340 ->
+// 282; the 48 kHz array 1285 -> 1193.)
+// The chunk's taps of the microphones and the signal window it needs (the
 // samples outside the segment zeroed) are staged in the warp's shared memory,
 // the taps as [microphone][k] rows copied with 128-bit loads when every RIR
 // row starts on a 16-byte boundary (n_S a multiple of 4; the chunk's first
@@ -29,14 +33,13 @@
 namespace {
 
 #define AU_R 4                       // outputs per lane
-#define AU_M 8                       // microphones per CTA
 #define AU_KC 128                    // taps per staged chunk
-#define AU_WARPS 4                   // warps per CTA (segments split round-robin)
 #define AU_TILE (32 * AU_R)          // outputs per CTA
 #define AU_XN (AU_TILE + AU_KC)      // signal samples per chunk (the last one is never used)
 
 static_assert(AU_R == 4 && AU_KC % 4 == 0, "the signal window is read as float4 groups of 4 taps");
 
+template <int AU_M>
 struct AuWarp {
     float4 h[AU_M][AU_KC / 4];       // taps of the chunk: [microphone][k / 4]
     float4 x[AU_XN / 4];             // signal window
@@ -62,16 +65,15 @@ __device__ __forceinline__ int au_start(int p, int n_x, int n_points, const int*
     return min(max(starts[p], 0), n_x);
 }
 
-template <bool VEC>   // 128-bit tap staging (16-byte aligned RIR rows)
-__global__ void __launch_bounds__(AU_WARPS * 32, 6) auralize_kernel(const float* __restrict__ x, int n_x,
-                                                                 const float* __restrict__ h, int n_points,
-                                                                 int n_mics, int n_s,
-                                                                 const int* __restrict__ starts,
-                                                                 float* __restrict__ y, int n_out)
+// VEC: 128-bit tap staging (16-byte aligned RIR rows); AU_M: microphones per CTA
+template <bool VEC, int AU_M, int AU_WARPS>
+__global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS == 4 ? 6 : 1)
+    auralize_kernel(const float* __restrict__ x, int n_x, const float* __restrict__ h, int n_points, int n_mics, int n_s,
+                    const int* __restrict__ starts, float* __restrict__ y, int n_out)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    AuWarp& W = reinterpret_cast<AuWarp*>(smem)[warp];
+    AuWarp<AU_M>& W = reinterpret_cast<AuWarp<AU_M>*>(smem)[warp];
     const long long T0 = (long long)blockIdx.x * AU_TILE;
     const int m0 = blockIdx.y * AU_M;
 
@@ -87,17 +89,29 @@ __global__ void __launch_bounds__(AU_WARPS * 32, 6) auralize_kernel(const float*
     if (s_lo <= s_hi) {
         const int p_lo = au_segment(s_lo, n_x, n_points, starts);
         const int p_hi = au_segment(s_hi, n_x, n_points, starts);
-        for (int p = p_lo + warp; p <= p_hi; p += AU_WARPS) {
-            const int a = au_start(p, n_x, n_points, starts);
-            const int b = max(a, p + 1 < n_points ? au_start(p + 1, n_x, n_points, starts) : n_x);
+        int turn = 0;   // chunks of the segments so far, modulo the warps
+        for (int p0 = p_lo; p0 <= p_hi; p0 += 32) {
+          // the bounds of 32 segments at once, a lane each
+          int a_l = 0, b_l = 0;
+          if (p0 + lane <= p_hi) {
+              a_l = au_start(p0 + lane, n_x, n_points, starts);
+              b_l = max(a_l, p0 + lane + 1 < n_points ? au_start(p0 + lane + 1, n_x, n_points, starts) : n_x);
+          }
+          for (int pp = 0; pp < min(32, p_hi - p0 + 1); ++pp) {
+            const int p = p0 + pp;
+            const int a = __shfl_sync(0xffffffffu, a_l, pp), b = __shfl_sync(0xffffffffu, b_l, pp);
             if (b <= a) continue;
             // taps linking [a, b) to the tile (the vector form starts on a multiple of 4)
             const long long k_lo = VEC ? (max(T0 - b + 1, 0ll) & ~3ll) : max(T0 - b + 1, 0ll);
             const long long k_hi = min(T0 + AU_TILE - 1 - a, (long long)n_s - 1);
+            if (k_hi < k_lo) continue;
             const float* hp = h + (long long)p * n_mics * n_s;
-            for (long long k0 = k_lo; k0 <= k_hi; k0 += AU_KC) {
+            const int n_ch = (int)((k_hi - k_lo) / AU_KC) + 1;
+            const int first = (warp - turn + AU_WARPS) % AU_WARPS;   // the warp's first chunk of this segment
+            turn = (turn + n_ch) % AU_WARPS;
+            for (long long k0 = k_lo + (long long)first * AU_KC; k0 <= k_hi; k0 += AU_WARPS * AU_KC) {
                 __syncwarp();
-                // taps k0 .. k0 + KC - 1 of the 8 microphones (0 past k_hi or past the array)
+                // taps k0 .. k0 + KC - 1 of the microphones (0 past k_hi or past the array)
                 if (VEC) {
                     for (int e = lane; e < AU_M * AU_KC / 4; e += 32) {   // 32 lanes: 512 contiguous bytes
                         const int m = e / (AU_KC / 4), kq = e % (AU_KC / 4);
@@ -154,6 +168,7 @@ __global__ void __launch_bounds__(AU_WARPS * 32, 6) auralize_kernel(const float*
                     xb4 = xa;
                 }
             }
+          }
         }
     }
 
@@ -177,27 +192,48 @@ __global__ void __launch_bounds__(AU_WARPS * 32, 6) auralize_kernel(const float*
     }
 }
 
-}  // namespace
-
-size_t ism_auralize_smem()
+template <bool VEC, int AU_M, int AU_WARPS>
+int launch_au(const float* x, int n_x, const float* h, int n_points, int n_mics, int n_s, const int* starts, float* y,
+              cudaStream_t s)
 {
-    const size_t stage = AU_WARPS * sizeof(AuWarp);
-    const size_t red = (size_t)AU_WARPS * AU_R * AU_M * 32 * sizeof(float);
-    return stage > red ? stage : red;
+    const long long n_out = (long long)n_x + n_s - 1;
+    const dim3 grid((unsigned)((n_out + AU_TILE - 1) / AU_TILE), (unsigned)((n_mics + AU_M - 1) / AU_M));
+    const size_t sm = std::max(AU_WARPS * sizeof(AuWarp<AU_M>), (size_t)AU_WARPS * AU_R * AU_M * 32 * sizeof(float));
+    static std::atomic<unsigned long long> opened{0};
+    const int rc = ism_open_smem((const void*)auralize_kernel<VEC, AU_M, AU_WARPS>, &opened);
+    if (rc) return rc;
+    auralize_kernel<VEC, AU_M, AU_WARPS><<<grid, AU_WARPS * 32, sm, s>>>(x, n_x, h, n_points, n_mics, n_s, starts, y,
+                                                                       (int)n_out);
+    return (int)cudaGetLastError();
 }
+
+template <bool VEC, int AU_M>
+int launch_au_m(const float* x, int n_x, const float* h, int n_points, int n_mics, int n_s, const int* starts, float* y,
+                cudaStream_t s)
+{
+    // 16 warps share a tile; 4 where segments are shorter than a chunk and there are tiles
+    // enough, since every warp goes through the bounds of all the tile's segments (3000
+    // segments of 16 samples, 445 tiles: 1455 us against 1786)
+    const long long tiles = (((long long)n_x + n_s - 1 + AU_TILE - 1) / AU_TILE) * ((n_mics + AU_M - 1) / AU_M);
+    return n_x / n_points < AU_KC && tiles >= 304
+               ? launch_au<VEC, AU_M, 4>(x, n_x, h, n_points, n_mics, n_s, starts, y, s)
+               : launch_au<VEC, AU_M, 16>(x, n_x, h, n_points, n_mics, n_s, starts, y, s);
+}
+
+}  // namespace
 
 int ism_launch_auralize(const float* x, int n_x, const float* h, int n_points, int n_mics, int n_s,
                         const int* starts, float* y, void* stream)
 {
-    const long long n_out = (long long)n_x + n_s - 1;
-    const dim3 grid((unsigned)((n_out + AU_TILE - 1) / AU_TILE), (unsigned)((n_mics + AU_M - 1) / AU_M));
-    const size_t sm = ism_auralize_smem();
+    cudaStream_t s = (cudaStream_t)stream;
     // 128-bit tap rows when every row starts on a 16-byte boundary
     const bool vec = (n_s % 4 == 0) && (((uintptr_t)h & 15u) == 0);
-    auto kern = vec ? auralize_kernel<true> : auralize_kernel<false>;
-    static std::atomic<unsigned long long> opened[2] = {{0}, {0}};
-    const int rc = ism_open_smem((const void*)kern, &opened[vec ? 1 : 0]);
-    if (rc) return rc;
-    kern<<<grid, AU_WARPS * 32, sm, (cudaStream_t)stream>>>(x, n_x, h, n_points, n_mics, n_s, starts, y, (int)n_out);
-    return (int)cudaGetLastError();
+#define AU_L(M)                                                                      \
+    return vec ? launch_au_m<true, M>(x, n_x, h, n_points, n_mics, n_s, starts, y, s) \
+               : launch_au_m<false, M>(x, n_x, h, n_points, n_mics, n_s, starts, y, s)
+    if (n_mics == 1) AU_L(1);
+    if (n_mics == 2) AU_L(2);
+    if (n_mics <= 4) AU_L(4);
+    AU_L(8);
+#undef AU_L
 }
