@@ -1,7 +1,7 @@
 // ism_adjoint.cu -- gradients of a loss through the image-source RIR: the
 // adjoint of eq. (1)-(6) (the paper computes forward RIRs only), per tap, for
-// windows other than exactly 32 taps (those take the fused Chebyshev adjoint
-// of ism_adjoint_cheb.cu), and the reduction of every job's gradients.
+// the short windows that the fused Chebyshev adjoint of ism_adjoint_cheb.cu does
+// not take, and the reduction of every job's gradients.
 //
 // The binned image lists of the forward pass (enumeration + counting sort)
 // are reused: one CTA per (RIR, tile of 8 delay bins), one warp per bin, as

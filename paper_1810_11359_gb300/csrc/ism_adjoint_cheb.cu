@@ -1,7 +1,7 @@
-// ism_adjoint_cheb.cu -- gradients of a loss through the image-source RIR for
-// a window of exactly 32 taps, through the Chebyshev expansion of the tap
-// functions that the forward FP32 form uses (the paper computes forward RIRs
-// only; the chain rule is that of eq. (1)-(6)).
+// ism_adjoint_cheb.cu -- gradients of a loss through the image-source RIR
+// through the Chebyshev expansion of the tap functions that the forward FP32
+// form uses (the paper computes forward RIRs only; the chain rule is that of
+// eq. (1)-(6)): windows of 32 taps with 9 terms (the text below), others with 11.
 //
 // With g_k = dLoss/dh[k], an image of integer delay b = 32 q + o - 1 and
 // fractional delay f has, per tap t = 0 .. 31 (sample k = 32 q - 16 + o + t,
@@ -30,24 +30,39 @@
 // warp order; the CTA's 12 sums go to the slot of its first bin (zeros to the
 // slots of its other bins), which the reduction kernel adds per RIR in bin
 // order: no atomics, bit-identical from run to run.
+//
+// Other windows (2 H taps, coefficients from the table that the geometry launch
+// fills).  The series has to follow the taps' derivatives too, in which the kink of
+// a window that ends inside a sample interval is far larger than in the taps
+// themselves: degree 10 keeps them to 2.3e-8 (rms over the taps) for windows of a
+// whole even number of taps and for any of ISM_ADJ_MIN_NW or more; shorter masked
+// windows keep the per-tap adjoint.  Fitting one room, 8 RIRs of 64 taps: geometry,
+// count, scan (3), scatter and per-tap adjoint 83 us -> geometry and this 26 us.
+#include <algorithm>
+
 #include "ism_shell.cuh"
 
 namespace {
 
 #define SA_B ISM_SHELL_BINS   // delay bins per CTA
 #define SA_WARPS 8            // warps per CTA (one per bin for the tables)
-#define SA_GV 3               // float4 per Gamma row (9 terms + 3 pad)
+#define SA_GV 3               // float4 per Gamma row (9 or 11 terms, padded)
 #define SA_NG 12              // gradient components: dp_r[3], dp_s[3], dbeta[6]
 
+template <int NT>
 __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const __grid_constant__ JobTable t,
                                                                           const float4* __restrict__ tbl,
                                                                           const float4* __restrict__ dtbl,
-                                                                          float* __restrict__ gpart)
+                                                                          const float* __restrict__ tabs,
+                                                                          float* __restrict__ gpart, int max_taps)
 {
+    constexpr bool PLAIN = NT == ISM_CHEB_N;   // 32 taps, coefficients in the parameter table
+    static_assert(NT <= 4 * SA_GV, "a Gamma row holds the terms");
     extern __shared__ __align__(16) unsigned char smem[];
     int jid, r, grp;
     if (!shell_cta(t, blockIdx.x, &jid, &r, &grp)) return;   // CTA-uniform
     const JobDev& J = t.j[jid];
+    if (J.adj_cheb != NT) return;   // another instantiation's job
     const int q0 = grp * SA_B;
     const int nb = min(SA_B, J.Q - q0);
     const int Nx = J.N[0], Ny = J.N[1];
@@ -59,9 +74,10 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     const int axis_pad = (t.max_axis_sum + 1) & ~1;
     const ShellTab T = shell_tab(smem, t.max_axis_sum);
     float4* X = reinterpret_cast<float4*>(smem) + axis_pad;   // x_n - x_r, dF/dbeta_lo, dF/dbeta_hi, d x_n / d x_s
-    float4* Gam = X + axis_pad;                                 // [bin][offset][SA_GV]: Gamma_0..8
-    float* gw = reinterpret_cast<float*>(Gam + SA_B * 32 * SA_GV);   // [bin][64]
-    float* red = gw + SA_B * 64;                                // [warp][SA_NG]
+    float4* Gam = X + axis_pad;                                 // [bin, offset][SA_GV]: Gamma_0 .. NT - 1
+    float4* ct = Gam + SA_B * 32 * SA_GV;                       // [tap][SA_GV]: coefficients (not PLAIN)
+    float* gw = reinterpret_cast<float*>(ct + (PLAIN ? 0 : max_taps * SA_GV));   // dLoss/dh from sample 32 q0 - H
+    float* red = gw + SA_B * 32 + max_taps;                     // [warp][SA_NG]
     int* rowpre = reinterpret_cast<int*>(red + SA_WARPS * SA_NG);
     int* rowy0 = rowpre + ((t.max_axis_sum + 4) & ~3);
     float4* recf = reinterpret_cast<float4*>(rowy0 + ((t.max_axis_sum + 4) & ~3));
@@ -76,29 +92,49 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
         shell_stage<true>(T, e, Tg[e], s2_magic);
         X[e] = Xg[e];
     }
-    // dLoss/dh over the windows of the CTA's bins (samples 32 q - 16 + P, P < 64; 0 outside [0, n_ism))
+    // dLoss/dh over the windows of the CTA's bins (bin q's: samples 32 q - H + P, P < 32 + 2 H; 0
+    // outside [0, n_ism))
+    const int H = PLAIN ? 16 : J.H;
     const float* go = J.grad_out + (long long)r * J.n_S;
-    for (int e = threadIdx.x; e < SA_B * 64; e += blockDim.x) {
-        const int q = q0 + e / 64;
-        const int k = ISM_SB * q - 16 + (e % 64);
-        gw[e] = (q < J.Q && k >= 0 && k < J.n_ism) ? go[k] : 0.0f;
+    for (int e = threadIdx.x; e < SA_B * 32 + 2 * H; e += blockDim.x) {
+        const int k = ISM_SB * q0 - H + e;
+        gw[e] = (k >= 0 && k < J.n_ism) ? go[k] : 0.0f;
     }
+    if (!PLAIN)
+        for (int e = threadIdx.x; e < 2 * H * 4 * SA_GV; e += blockDim.x) {
+            const int i = e % (4 * SA_GV), tt = e / (4 * SA_GV);
+            reinterpret_cast<float*>(ct)[e] = i < NT ? tabs[J.lut_base + i * 32 * J.slots + tt] : 0.0f;
+        }
     __syncthreads();
-    {   // Gamma_i(q0 + warp, o = lane): 9 dot products of length 32 with the tap coefficients
-        const float* gwb = gw + warp * 64;
-        float acc[ISM_CHEB_N];
+    {   // Gamma_i(q0 + warp, o = lane): NT dot products of length 2 H with the tap coefficients
+        const float* gwb = gw + warp * 32 + lane;
+        float acc[4 * SA_GV];
 #pragma unroll
-        for (int i = 0; i < ISM_CHEB_N; ++i) acc[i] = 0.0f;
+        for (int i = 0; i < 4 * SA_GV; ++i) acc[i] = 0.0f;
+        if constexpr (PLAIN) {
 #pragma unroll
-        for (int tt = 0; tt < 32; ++tt) {
-            const float gk = gwb[lane + tt];
+            for (int tt = 0; tt < 32; ++tt) {
+                const float gk = gwb[tt];
 #pragma unroll
-            for (int i = 0; i < ISM_CHEB_N; ++i) acc[i] = __fmaf_rn(t.cheb[tt * ISM_CHEB_N + i], gk, acc[i]);
+                for (int i = 0; i < NT; ++i) acc[i] = __fmaf_rn(t.cheb[tt * ISM_CHEB_N + i], gk, acc[i]);
+            }
+        } else {
+#pragma unroll 4
+            for (int tt = 0; tt < 2 * H; ++tt) {
+                const float gk = gwb[tt];
+#pragma unroll
+                for (int v = 0; v < SA_GV; ++v) {
+                    const float4 c = ct[tt * SA_GV + v];
+                    acc[4 * v] = __fmaf_rn(c.x, gk, acc[4 * v]);
+                    acc[4 * v + 1] = __fmaf_rn(c.y, gk, acc[4 * v + 1]);
+                    acc[4 * v + 2] = __fmaf_rn(c.z, gk, acc[4 * v + 2]);
+                    if (4 * v + 3 < NT) acc[4 * v + 3] = __fmaf_rn(c.w, gk, acc[4 * v + 3]);
+                }
+            }
         }
         float4* row = Gam + (warp * 32 + lane) * SA_GV;
-        row[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        row[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-        row[2] = make_float4(acc[8], 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int v = 0; v < SA_GV; ++v) row[v] = make_float4(acc[4 * v], acc[4 * v + 1], acc[4 * v + 2], acc[4 * v + 3]);
     }
 
     // exact delays b owned by this CTA: [b_lo, b_hi), b <= n_ism + 14 (later taps miss [0, n_ism))
@@ -115,7 +151,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
                          [&](int bl, float f, float rs, const float4& cf, int col, int ez, const float4& tz) {
         const float4* Gr = Gam + bl * SA_GV;   // [bin][offset], 32 offsets per bin
         const float4 g0 = Gr[0], g1 = Gr[1], g2 = Gr[2];
-        const float Gb[ISM_CHEB_N] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w, g2.x};
+        const float Gb[4 * SA_GV] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w, g2.x, g2.y, g2.z, g2.w};
         // ga = sum_i Gamma_i T_i(u), gd = sum_i Gamma_i T_i'(u)
         const float uu = __fmaf_rn(2.0f, f, -1.0f);
         const float u2 = uu + uu;
@@ -123,7 +159,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
         float gd = Gb[1];
         float tp = 1.0f, tc = uu, dp = 0.0f, dc = 1.0f;
 #pragma unroll
-        for (int i = 2; i < ISM_CHEB_N; ++i) {
+        for (int i = 2; i < NT; ++i) {
             const float tn = __fmaf_rn(u2, tc, -tp);
             const float dn = __fmaf_rn(u2, dc, __fmaf_rn(2.0f, tc, -dp));   // T_i' = 2 T_(i-1) + 2 u T_(i-1)' - T_(i-2)'
             const float gi = Gb[i];
@@ -176,13 +212,26 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     for (int e = threadIdx.x; e < (nb - 1) * SA_NG; e += blockDim.x) dst[SA_NG + e] = 0.0f;
 }
 
-size_t shell_adjoint_smem(const JobTable& t)
+template <int NT>
+int launch_adj_cheb(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s, int max_taps)
 {
     const size_t axis_pad = (size_t)((t.max_axis_sum + 1) & ~1);
     const size_t rows = (size_t)((t.max_axis_sum + 4) & ~3);
-    return 2 * axis_pad * sizeof(float4) + (size_t)SA_B * 32 * SA_GV * sizeof(float4) +
-           (size_t)SA_B * 64 * sizeof(float) + (size_t)SA_WARPS * SA_NG * sizeof(float) + 2 * rows * sizeof(int) +
-           (size_t)SA_WARPS * 32 * (sizeof(float4) + sizeof(int2) + sizeof(int)) + (size_t)SA_WARPS * SHELL_MW * sizeof(unsigned);
+    const size_t sm = 2 * axis_pad * sizeof(float4) + (size_t)SA_B * 32 * SA_GV * sizeof(float4) +
+                      (NT == ISM_CHEB_N ? 0 : (size_t)max_taps * SA_GV * sizeof(float4)) +
+                      (size_t)(SA_B * 32 + max_taps) * sizeof(float) + (size_t)SA_WARPS * SA_NG * sizeof(float) +
+                      2 * rows * sizeof(int) + (size_t)SA_WARPS * 32 * (sizeof(float4) + sizeof(int2) + sizeof(int)) +
+                      (size_t)SA_WARPS * SHELL_MW * sizeof(unsigned);
+    static std::atomic<unsigned long long> opened{0};
+    int rc = ism_open_smem((const void*)shell_adjoint_kernel<NT>, &opened);
+    if (rc) return rc;
+    cudaError_t e = cudaFuncSetAttribute(shell_adjoint_kernel<NT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         cudaSharedmemCarveoutMaxShared);   // 4 CTAs of ~32 KB per SM
+    if (e != cudaSuccess) return (int)e;
+    shell_adjoint_kernel<NT><<<(unsigned)p.shell_ctas, SA_WARPS * 32, sm, s>>>(
+        t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<const float4*>(ws + p.dtbl_off),
+        reinterpret_cast<const float*>(ws + p.lut_off), reinterpret_cast<float*>(ws + p.gpart_off), max_taps);
+    return (int)cudaGetLastError();
 }
 
 }  // namespace
@@ -191,16 +240,16 @@ int ism_launch_adjoint_cheb(const JobTable& t, const WsPlan& p, char* ws, void* 
 {
     *launched = 0;
     if (p.shell_ctas <= 0) return 0;
-    const size_t sm = shell_adjoint_smem(t);
-    static std::atomic<unsigned long long> opened{0};
-    int rc = ism_open_smem((const void*)shell_adjoint_kernel, &opened);
-    if (rc) return rc;
-    cudaError_t e = cudaFuncSetAttribute(shell_adjoint_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         cudaSharedmemCarveoutMaxShared);   // 4 CTAs of ~32 KB per SM
-    if (e != cudaSuccess) return (int)e;
-    shell_adjoint_kernel<<<(unsigned)p.shell_ctas, SA_WARPS * 32, sm, (cudaStream_t)stream>>>(
-        t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<const float4*>(ws + p.dtbl_off),
-        reinterpret_cast<float*>(ws + p.gpart_off));
-    *launched = 1;
-    return (int)cudaGetLastError();
+    bool plain = false, wide = false;
+    int max_taps = 32;   // (a multiple of 4: the tables behind the window are 16-byte aligned)
+    for (int i = 0; i < t.n_jobs; ++i) {
+        plain |= t.j[i].adj_cheb == ISM_CHEB_N;
+        if (t.j[i].adj_cheb != ISM_CHEB_AW) continue;
+        wide = true;
+        max_taps = std::max(max_taps, (2 * t.j[i].H + 3) & ~3);
+    }
+    int rc = 0;
+    if (plain) rc = launch_adj_cheb<ISM_CHEB_N>(t, p, ws, (cudaStream_t)stream, 32), ++*launched;
+    if (!rc && wide) rc = launch_adj_cheb<ISM_CHEB_AW>(t, p, ws, (cudaStream_t)stream, max_taps), ++*launched;
+    return rc;
 }

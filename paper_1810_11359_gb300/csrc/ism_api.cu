@@ -306,9 +306,13 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
             // images costs more than adding every image's taps on its own
             J.sparse = ((prec == ISM_PREC_FP32 || prec == ISM_PREC_FP32_DIRECT) && !backward && !J.use_cheb &&
                         per_bin < 128.0) ? 1 : 0;
-            // backward: a 32-tap window always takes the fused Chebyshev adjoint (an
-            // image costs two degree-8 sums there, against 32 tap derivatives)
-            J.adj_cheb = (backward && v.Nw == 32.0 && v.H == 16 && v.slots == 1) ? 1 : 0;
+            // backward: the fused Chebyshev adjoint for the windows whose derivative its series
+            // follows (an image costs two degree-8 or -10 sums there, against the derivatives
+            // of all its taps, and no count, scan and scatter come before)
+            J.adj_cheb = 0;
+            if (backward && taps32) J.adj_cheb = ISM_CHEB_N;
+            else if (backward && (v.Nw == 2.0 * v.H ? v.Nw >= ISM_CHEB_MIN_NW : v.Nw >= ISM_ADJ_MIN_NW))
+                J.adj_cheb = ISM_CHEB_AW;
             // the other forward jobs with a 32-tap window, in every tap arithmetic: every tap
             // evaluated, the images enumerated by the CTA that accumulates them (no ids, no
             // sort); the value is the shell's thickness in bins: 32 for sparse bins, 8 for dense ones
@@ -370,10 +374,10 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
         if (prec == ISM_PREC_LUT) lut += (long long)(ism_lut_phases(J.slots) + 1) * 32 * J.slots;
         // texture form: each table starts on a 512-byte boundary (texture base alignment)
         if (prec == ISM_PREC_LUT_TEX) lut += ((long long)(ism_lut_phases(J.slots) + 1) * 32 * J.slots + 127) / 128 * 128;
-        if (J.use_cheb == ISM_CHEB_NW) {   // one coefficient table per window length
+        if (J.use_cheb == ISM_CHEB_NW || J.adj_cheb == ISM_CHEB_AW) {   // one coefficient table per window length
             J.lut_base = p.cheb_tabs * ISM_CHEB_TAB;
             for (int k = 0; k < i; ++k)
-                if (t.j[k].use_cheb == J.use_cheb && t.j[k].Nw == J.Nw) {
+                if (t.j[k].use_cheb == J.use_cheb && t.j[k].adj_cheb == J.adj_cheb && t.j[k].Nw == J.Nw) {
                     J.lut_base = t.j[k].lut_base;
                     break;
                 }

@@ -48,7 +48,9 @@
 #define ISM_CHEB_NF 8             // Chebyshev terms of the forward's moments (degree 7)
 #define ISM_CHEB_NW 10            // the same for windows other than 32 taps (degree 9)
 #define ISM_CHEB_MIN_NW 16        // shortest window whose taps the series reproduces (see ism_accum_cheb.cu)
+#define ISM_CHEB_AW 11            // terms of the adjoint for windows other than 32 taps (degree 10)
 #define ISM_CHEB_MAX 12           // terms of any of them, at most
+#define ISM_ADJ_MIN_NW 80         // windows that end inside a sample interval: shortest for the fused adjoint
 #define ISM_CHEB_TAB 4096         // floats of a coefficient table in the workspace: [term][32 slots]
 #define ISM_CHEB_TAB_CTAS 32      // CTAs that fill one (8 taps each)
 #define ISM_SHELL_BINS 8          // delay bins per CTA of the fused Chebyshev accumulation
@@ -90,7 +92,7 @@ struct JobDev {
     int use_cheb;             // FP32 accumulation through Chebyshev moments: the terms (0: not this form)
     int shell_groups;         // fused Chebyshev CTAs per RIR (ISM_SHELL_BINS bins each; 0 otherwise)
     int sparse;               // direct FP32 form, few images per bin: no sort, each image's taps added at once
-    int adj_cheb;             // backward: fused Chebyshev adjoint (32-tap window; shell_groups CTAs per RIR)
+    int adj_cheb;             // backward: fused Chebyshev adjoint: the terms (0: not this form)
     int rir_index0;           // RIR index of the job's first RIR in its caller's job (noise counter)
     uint64_t seed;
     const float* pos_src;
