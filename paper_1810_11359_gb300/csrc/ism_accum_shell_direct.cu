@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
     const float rscale = (PREC == PREC_FP16) ? J.half_scale : 1.0f;
     const float dscale = (PREC == PREC_FP16) ? 1.0f / J.half_scale : 1.0f;
     const float f_lo = HALF ? 0x1p-13f : 0x1p-60f;
-    const float f_hi = HALF ? 1.0f - 0x1p-13f : 1.0f;
+    const float f_hi = HALF ? 1.0f - 0x1p-13f : 1.0f - 0x1p-24f;   // (f = 1 is a fraction of shell_delay's)
     const float* lut = PREC == PREC_LUT ? lut_g + J.lut_base + lane : nullptr;
 
     // (the shell's window starts at sample 32 q0 - 16: tap 0 of an image of integer delay
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
                 float amp = SPLIT ? cf.z * tz.z * rs : cf.z * tz.z * J.amp_scale * rs;
                 if (alpha != 1.0f)   // polar pattern: cos(theta) = o . (x_n - x_r) / d
                     amp *= __fmaf_rn(1.0f - alpha, __fmaf_rn(orient.z, tz.w, Wo[col]) * rs, alpha);
-                f = fminf(fmaxf(f, f_lo), f_hi);   // keeps j - f away from 0 (the reciprocal of the tap j = 0)
+                f = fminf(fmaxf(f, f_lo), f_hi);   // keeps j - f away from 0 (the reciprocals of the taps j = 0 and 1)
                 if constexpr (PREC == PREC_LUT) {
                     // eq. (9): rows floor(f Q) and + 1 of the polyphase table, weights A (1 - phi), A phi
                     const float u = f * (float)LQ;   // exact: LQ is a power of two

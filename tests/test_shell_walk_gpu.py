@@ -58,3 +58,21 @@ def test_adjoint(c):
     for a, b in zip(got, ref):
         a = a.cpu().numpy().astype(np.float64).reshape(-1)
         assert np.max(np.abs(a - b)) <= 1e-4 * np.max(np.abs(b))
+
+
+@pytest.mark.parametrize("eps", [0.0, 1e-12, 1e-10, 1e-9, 5e-9, 1e-8, 3e-8, 5e-8, -1e-9, -3e-8])
+@pytest.mark.parametrize("prec", ["fp32", "fp32_direct"])
+def test_delays_next_to_an_integer(eps, prec):
+    """Direct paths of 10 - eps samples (k = 1 sample per metre): a fraction that rounds to 1."""
+    fs, c, Tw = 343.0, 343.0, 32 / 343.0
+    dx = np.float64(np.float32(10.0) - np.float32(2.0 ** -18))   # the FP32 grid of y sets s to ~1e-12
+    dy = np.float32(np.sqrt((10.0 - eps) ** 2 - dx * dx))
+    L, beta, N = [40.0, 38.0, 36.0], np.full(6, 0.5, np.float32), [5, 5, 5]
+    ps = np.array([[8.0, 2.0 ** -7, 16.0]], np.float32)
+    pr = np.array([[8.0 + dx, 2.0 ** -7 + dy, 16.0]], np.float32)
+    h = ism.ism_simulate(L, beta, torch.from_numpy(ps).cuda(), torch.from_numpy(pr).cuda(), N, 0.25, fs, Tw=Tw, c=c, prec=prec)
+    got = h.cpu().numpy().astype(np.float64)[0, 0]
+    assert np.all(np.isfinite(got))
+    ref = oracle.rir(L, beta.astype(np.float64), c, fs, float(np.float32(Tw)), ps[0].astype(np.float64),
+                     pr[0].astype(np.float64), N, got.size)
+    assert np.max(np.abs(got - ref)) <= 1e-5 * np.max(np.abs(ref))
