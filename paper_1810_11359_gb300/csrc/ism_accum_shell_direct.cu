@@ -41,31 +41,6 @@
 
 namespace {
 
-// Two FP32 values in one 64-bit register pair, and the packed FP32 operations of
-// sm_100-class GPUs on them (both lanes rounded as the scalar operations are).
-__device__ __forceinline__ unsigned long long sd_pack(float a, float b)
-{
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void sd_unpack(unsigned long long r, float& a, float& b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ unsigned long long sd_fma2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long sd_mul2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 #define SD_B ISM_SD_BINS             // delay bins per CTA, at most
 #define SD_WARPS 8                   // warps per CTA
 #define SD_RING 64                   // staged image records per warp (a ring; 32 are added at once)
@@ -156,8 +131,8 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
     const float xj = sg * (float)j, nsg = -sg;
     float Sj, Cj;
     sincospif((float)j * (2.0f / 32.0f), &Sj, &Cj);
-    const unsigned long long xj2 = sd_pack(xj, xj), nsg2 = sd_pack(nsg, nsg), Cj2 = sd_pack(Cj, Cj),
-                             Sj2 = sd_pack(Sj, Sj);
+    const unsigned long long xj2 = pk_pack(xj, xj), nsg2 = pk_pack(nsg, nsg), Cj2 = pk_pack(Cj, Cj),
+                             Sj2 = pk_pack(Sj, Sj);
     const float twopi_Nw = 6.283185307179586f / 32.0f, inv2Nw = 2.0f / 32.0f;
     uint32_t C2 = 0, S2 = 0;
     if constexpr (HALF) {
@@ -200,19 +175,19 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
             const int2 pp = sp2[k];
             float va, vb;
             if constexpr (PREC == PREC_FP32) {
-                const unsigned long long x2 = sd_fma2(nsg2, fa.x, xj2);
-                const unsigned long long w2 = sd_fma2(Cj2, fb.x, sd_fma2(Sj2, fb.y, fa.y));
+                const unsigned long long x2 = pk_fma(nsg2, fa.x, xj2);
+                const unsigned long long w2 = pk_fma(Cj2, fb.x, pk_fma(Sj2, fb.y, fa.y));
                 float xa, xb;
-                sd_unpack(x2, xa, xb);
-                sd_unpack(sd_mul2(w2, sd_pack(ism_rcp(xa), ism_rcp(xb))), va, vb);
+                pk_unpack(x2, xa, xb);
+                pk_unpack(pk_mul(w2, pk_pack(ism_rcp(xa), ism_rcp(xb))), va, vb);
             } else if constexpr (HALF) {
                 // x in FP32, then the window and the reciprocal in packed 16-bit arithmetic;
                 // the products of two 16-bit values are exact in FP32
                 float xa, xb, Pa, Pb, Pca, Pcb, Psa, Psb;
-                sd_unpack(sd_fma2(nsg2, fa.x, xj2), xa, xb);
-                sd_unpack(fa.y, Pa, Pb);
-                sd_unpack(fb.x, Pca, Pcb);
-                sd_unpack(fb.y, Psa, Psb);
+                pk_unpack(pk_fma(nsg2, fa.x, xj2), xa, xb);
+                pk_unpack(fa.y, Pa, Pb);
+                pk_unpack(fb.x, Pca, Pcb);
+                pk_unpack(fb.y, Psa, Psb);
                 const uint32_t w = fma2<PREC>(C2, pack2<PREC>(Pca, Pcb), fma2<PREC>(S2, pack2<PREC>(Psa, Psb),
                                                                                    pack2<PREC>(Pa, Pb)));
                 va = 0.0f;
@@ -222,17 +197,17 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
                 vb *= dscale;
             } else if constexpr (PREC == PREC_LUT) {
                 float w0a, w0b, w1a, w1b, ra, rb;
-                sd_unpack(fa.x, w0a, w0b);
-                sd_unpack(fa.y, w1a, w1b);
-                sd_unpack(fb.x, ra, rb);
+                pk_unpack(fa.x, w0a, w0b);
+                pk_unpack(fa.y, w1a, w1b);
+                pk_unpack(fb.x, ra, rb);
                 const float* pa = lut + __float_as_int(ra);
                 const float* pb = lut + __float_as_int(rb);
                 va = __fmaf_rn(w1a, __ldg(pa + 32), w0a * __ldg(pa));
                 vb = __fmaf_rn(w1b, __ldg(pb + 32), w0b * __ldg(pb));
             } else {   // PREC_TEX: one filtered fetch per tap
                 float Aa, Ab, ya, yb;
-                sd_unpack(fa.x, Aa, Ab);
-                sd_unpack(fa.y, ya, yb);
+                pk_unpack(fa.x, Aa, Ab);
+                pk_unpack(fa.y, ya, yb);
                 const cudaTextureObject_t tex = (cudaTextureObject_t)J.lut_tex;
                 va = Aa * tex2D<float>(tex, (float)lane + 0.5f, ya);
                 vb = Ab * tex2D<float>(tex, (float)lane + 0.5f, yb);

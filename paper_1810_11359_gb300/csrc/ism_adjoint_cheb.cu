@@ -27,9 +27,9 @@
 // (lane = offset o) from dLoss/dh over the bin's 64-sample window; then every
 // lane accumulates the gradients of the images it is handed in 12 registers.
 // The lanes' sums are reduced by a fixed butterfly per warp and the warps in
-// warp order; the CTA's 12 sums go to the slot of its first bin (zeros to the
-// slots of its other bins), which the reduction kernel adds per RIR in bin
-// order: no atomics, bit-identical from run to run.
+// warp order; the CTA's 12 sums go to the slot of its first bin, and the
+// reduction kernel adds the shells' slots per RIR in a fixed order: no atomics,
+// bit-identical from run to run.
 //
 // Other windows (2 H taps, coefficients from the table that the geometry launch
 // fills).  The series has to follow the taps' derivatives too, in which the kink of
@@ -209,7 +209,6 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
         for (int w = 1; w < SA_WARPS; ++w) v += red[w * SA_NG + threadIdx.x];
         dst[threadIdx.x] = v;
     }
-    for (int e = threadIdx.x; e < (nb - 1) * SA_NG; e += blockDim.x) dst[SA_NG + e] = 0.0f;
 }
 
 template <int NT>

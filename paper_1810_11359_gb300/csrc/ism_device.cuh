@@ -114,9 +114,11 @@ __device__ __forceinline__ float ism_exp2_neg(ff g, int i)
     const float p = __fmul_rn(g.hi, fi);
     if (!(p < 256.0f)) return 0.0f;   // below 2^-255: zero in FP32 (also catches an infinite rate)
     const float pe = __fmaf_rn(g.lo, fi, __fmaf_rn(g.hi, fi, -p));
-    const float n = rintf(p);
-    const float r = __fadd_rn(__fsub_rn(p, n), pe);
-    return ldexpf(exp2f(-r), -(int)n);
+    const float t = __fadd_rn(p, 12582912.0f);   // 1.5 2^23 + n, its bits hold n
+    const float r = __fadd_rn(__fsub_rn(p, __fsub_rn(t, 12582912.0f)), pe);
+    const int n = __float_as_int(t) - 0x4B400000;
+    const float e = exp2f(-r);
+    return n <= 125 ? __int_as_float(__float_as_int(e) - (n << 23)) : ldexpf(e, -n);
 }
 
 // Approximate reciprocal and reciprocal square root on the special-function
@@ -234,38 +236,85 @@ __device__ __forceinline__ uint4 ism_philox(uint4 c, uint32_t k0, uint32_t k1)
 //         ln m = 2t + t^3 (2/3 + t^2 (2/5 + t^2 (2/7 + t^2 (2/9 + t^2 2/11))))
 //         ln r = e ln2_hi + (e ln2_lo + ln m)
 //   z = (sqrt(3)/pi) ln r                           unit-variance logistic
-__device__ __forceinline__ float ism_uniform(uint32_t x)
+// Two FP32 values in one 64-bit register pair, and the packed FP32 operations of
+// sm_100-class GPUs on them (both halves rounded as the scalar operations are).
+__device__ __forceinline__ unsigned long long pk_pack(float a, float b)
 {
-    float m = __uint2float_rn(x >> 9);
-    return __fmul_rn(__fadd_rn(m, 0.5f), 0x1p-23f);
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void pk_unpack(unsigned long long r, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ unsigned long long pk_fma(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pk_mul(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pk_add(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pk_all(float a) { return pk_pack(a, a); }
+
+// -(a / b), correctly rounded, for quotients far from the ends of the FP32 range:
+// Markstein's sequence (IBM J. Res. Dev. 34, 1990) -- a reciprocal refined once, the
+// quotient and its exact remainder by FMAs -- with every sign turned, so that no
+// negation is an instruction.  Checked against / for every argument that the
+// noise gives it (all 2^23 uniforms; tests).
+__device__ __forceinline__ unsigned long long pk_neg_div(unsigned long long a, unsigned long long b)
+{
+    float b0, b1;
+    pk_unpack(b, b0, b1);
+    unsigned long long ny = pk_pack(ism_rcp(-b0), ism_rcp(-b1));   // -1 / b, one ulp
+    ny = pk_fma(ny, pk_fma(b, ny, pk_all(1.0f)), ny);
+    const unsigned long long nq = pk_mul(a, ny);
+    return pk_fma(pk_fma(b, nq, a), ny, nq);
 }
 
-__device__ __forceinline__ float ism_ln_spec(float x)
+// The transform of two words: its operations in its order, each rounded on its own, two
+// at a time.  (The uniform and the exponents come from additions to 2^23 and
+// 1.5 2^23 whose results are exact, not from the conversion unit.)  Tail of 512 RIRs of
+// 43,200 samples: 72 us one at a time with the compiler's division, XX us.
+__device__ __forceinline__ float2 ism_logistic2(uint32_t x0, uint32_t x1)
 {
-    uint32_t bits = __float_as_uint(x);
-    int e = (int)((bits >> 23) & 0xFFu) - 127;
-    float m = __uint_as_float((bits & 0x007FFFFFu) | 0x3F800000u);
-    if (m > 1.41421353816986083984375f) {
-        m = __fmul_rn(m, 0.5f);
-        e += 1;
-    }
-    float t = __fdiv_rn(__fsub_rn(m, 1.0f), __fadd_rn(m, 1.0f));
-    float t2 = __fmul_rn(t, t);
-    float p = __fmaf_rn(t2, 2.0f / 11.0f, 2.0f / 9.0f);
-    p = __fmaf_rn(t2, p, 2.0f / 7.0f);
-    p = __fmaf_rn(t2, p, 2.0f / 5.0f);
-    p = __fmaf_rn(t2, p, 2.0f / 3.0f);
-    float t3 = __fmul_rn(t, t2);
-    float lnm = __fmaf_rn(t3, p, __fmul_rn(2.0f, t));
-    float ef = __int2float_rn(e);
-    return __fmaf_rn(ef, 0.693145751953125f, __fmaf_rn(ef, 1.428606765330187e-06f, lnm));
-}
-
-__device__ __forceinline__ float ism_logistic(uint32_t x)
-{
-    float u = ism_uniform(x);
-    float r = __fdiv_rn(u, __fsub_rn(1.0f, u));
-    return __fmul_rn(0.5513288974761963f, ism_ln_spec(r));
+    // u = (n + 1/2) 2^-23 = (2^23 + n) 2^-23 - (1 - 2^-24), n = x >> 9
+    const unsigned long long f = pk_pack(__uint_as_float((x0 >> 9) | 0x4B000000u), __uint_as_float((x1 >> 9) | 0x4B000000u));
+    const unsigned long long u = pk_fma(f, pk_all(0x1p-23f), pk_all(-(1.0f - 0x1p-24f)));
+    float r0, r1;   // -u / (1 - u)
+    pk_unpack(pk_neg_div(u, pk_fma(u, pk_all(-1.0f), pk_all(1.0f))), r0, r1);
+    // |r| = m 2^e, m in (sqrt(1/2), sqrt(2)]: a carry out of the mantissa above that of sqrt(2)
+    const uint32_t i0 = __float_as_uint(r0), i1 = __float_as_uint(r1);
+    const uint32_t c0 = i0 + 0x4AFB0Cu, c1 = i1 + 0x4AFB0Cu;
+    const unsigned long long m = pk_pack(__uint_as_float(i0 - (c0 & 0xFF800000u) + 0x3F800000u),
+                                         __uint_as_float(i1 - (c1 & 0xFF800000u) + 0x3F800000u));
+    // 1.5 2^23 + e (the shifted word is 256 + 127 + e), then -e
+    const unsigned long long eb = pk_pack(__uint_as_float((c0 >> 23) + (0x4B400000u - 383u)),
+                                          __uint_as_float((c1 >> 23) + (0x4B400000u - 383u)));
+    const unsigned long long ne = pk_fma(eb, pk_all(-1.0f), pk_all(12582912.0f));
+    const unsigned long long nt = pk_neg_div(pk_add(m, pk_all(-1.0f)), pk_add(m, pk_all(1.0f)));   // -(m - 1) / (m + 1)
+    const unsigned long long t2 = pk_mul(nt, nt);
+    unsigned long long p = pk_fma(t2, pk_all(2.0f / 11.0f), pk_all(2.0f / 9.0f));
+    p = pk_fma(t2, p, pk_all(2.0f / 7.0f));
+    p = pk_fma(t2, p, pk_all(2.0f / 5.0f));
+    p = pk_fma(t2, p, pk_all(2.0f / 3.0f));
+    const unsigned long long nln = pk_fma(pk_mul(nt, t2), p, pk_mul(pk_all(2.0f), nt));   // -ln m
+    const unsigned long long nl =
+        pk_fma(ne, pk_all(0.693145751953125f), pk_fma(ne, pk_all(1.428606765330187e-06f), nln));
+    float z0, z1;
+    pk_unpack(pk_mul(pk_all(-0.5513288974761963f), nl), z0, z1);
+    return make_float2(z0, z1);
 }
 
 // Noise of sample k of RIR `rir`: word k mod 4 of Philox(counter (k/4, rir,
@@ -274,5 +323,6 @@ __device__ __forceinline__ float ism_logistic(uint32_t x)
 __device__ __forceinline__ float4 ism_noise_block(uint64_t seed, uint32_t rir, uint32_t blk)
 {
     uint4 w = ism_philox(make_uint4(blk, rir, 0u, 0u), (uint32_t)seed, (uint32_t)(seed >> 32));
-    return make_float4(ism_logistic(w.x), ism_logistic(w.y), ism_logistic(w.z), ism_logistic(w.w));
+    const float2 a = ism_logistic2(w.x, w.y), b = ism_logistic2(w.z, w.w);
+    return make_float4(a.x, a.y, b.x, b.y);
 }

@@ -141,15 +141,22 @@ __global__ void __launch_bounds__(256) tail_kernel(const __grid_constant__ JobTa
     const float sqA = sqrtf(amp[J.rir_base + r]);
     // Sabine envelope of a block of 4 samples from its first one: e_(k+d) = e_k R_d,
     // R_d = 2^(-hg d) for d = 1 .. 3 (each within 2 ulp, the product rounded once more:
-    // a few 1e-7 of the sample, see ism_exp2_neg)
-    __shared__ ff g2_s;
-    __shared__ float R_s[4];
-    if (threadIdx.x == 0) g2_s = ism_job_g2(J);
-    __syncthreads();
-    const ff hg = {0.5f * g2_s.hi, 0.5f * g2_s.lo};   // amplitude: half the power's rate (exact)
-    if (threadIdx.x < 4) R_s[threadIdx.x] = ism_exp2_neg(hg, (int)threadIdx.x);
-    __syncthreads();
-    const float R1 = R_s[1], R2 = R_s[2], R3 = R_s[3];
+    // a few 1e-7 of the sample, see ism_exp2_neg).  A lane each and shuffles: no barrier
+    // (two of them were a fifth of this short kernel's stalls), but for the FP64 rate of
+    // coefficients in device memory.
+    ff g2;
+    if (J.beta_dev) {   // CTA-uniform
+        __shared__ ff g2_s;
+        if (threadIdx.x == 0) g2_s = ism_job_g2(J);
+        __syncthreads();
+        g2 = g2_s;
+    } else {
+        g2 = {J.g2, J.g2_lo};
+    }
+    const ff hg = {0.5f * g2.hi, 0.5f * g2.lo};   // amplitude: half the power's rate (exact)
+    const float Rd = ism_exp2_neg(hg, (int)threadIdx.x & 3);
+    const float R1 = __shfl_sync(0xffffffffu, Rd, 1), R2 = __shfl_sync(0xffffffffu, Rd, 2),
+                R3 = __shfl_sync(0xffffffffu, Rd, 3);
     const bool lj = J.envelope == ISM_ENVELOPE_LJ;
     const float* envt = env + J.env_base - J.env_k0;   // sqrt(E(t_k) / E(t0)), k >= env_k0
     float* out = J.out + (long long)r * J.n_S;
