@@ -200,6 +200,16 @@ __device__ __forceinline__ void mixed_fma2(float& da, float& db, uint32_t w, uin
     }
 }
 
+// d + lo(w) lo(r) (HI: of the high halves), one rounding to FP32.
+template <int PREC, bool HI>
+__device__ __forceinline__ float mixed_fma(float d, uint32_t w, uint32_t r)
+{
+    const uint16_t a = (uint16_t)(HI ? w >> 16 : w), b = (uint16_t)(HI ? r >> 16 : r);
+    if constexpr (PREC == PREC_FP16) asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(d) : "h"(a), "h"(b));
+    else asm("fma.rn.f32.bf16 %0, %1, %2, %0;" : "+f"(d) : "h"(a), "h"(b));
+    return d;
+}
+
 // Rotates the run total D (lane = tap) into the window (lane = position);
 // `scale` undoes the record scaling of the FP16 form (a power of two).
 template <int SLOTS, bool SCALED>

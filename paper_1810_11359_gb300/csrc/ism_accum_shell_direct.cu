@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
         C2 = pack2<PREC>(Cj, Cj);
         S2 = pack2<PREC>(Sj, Sj);
     }
-    // FP16 records are scaled by 2^e (undone, exactly, on each product); f is kept away
+    // FP16 records are scaled by 2^e (undone, exactly, on the window's sums); f is kept away
     // from 0 and 1 in the packed forms so that the packed reciprocal stays finite
     const float rscale = (PREC == PREC_FP16) ? J.half_scale : 1.0f;
     const float dscale = (PREC == PREC_FP16) ? 1.0f / J.half_scale : 1.0f;
@@ -159,7 +159,19 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
     const ulonglong2* st2 = reinterpret_cast<const ulonglong2*>(stage);
     const int2* sp2 = reinterpret_cast<const int2*>(spos);
     int head = 0, n_st = 0;   // (warp-uniform) first pair of the ring not yet added; records waiting
+    // FP16X2 / BF16X2: {f_a, f_b}, then the pairs {P_a, P_b}, {Pc_a, Pc_b}, {Ps_a, Ps_b} in 16
+    // bits each, converted once by the lane that found the image instead of by all 32.
     auto put = [&](int slot, const float4& rc, int pos) {
+        if constexpr (HALF) {
+            float* sl = reinterpret_cast<float*>(stage) + 8 * (slot >> 1);
+            sl[slot & 1] = rc.x;
+            uint16_t* hs = reinterpret_cast<uint16_t*>(sl + 2) + (slot & 1);
+            hs[0] = (uint16_t)pack2<PREC>(rc.y, 0.0f);
+            hs[2] = (uint16_t)pack2<PREC>(rc.z, 0.0f);
+            hs[4] = (uint16_t)pack2<PREC>(rc.w, 0.0f);
+            spos[slot] = pos;
+            return;
+        }
         float* sl = reinterpret_cast<float*>(stage) + 8 * (slot >> 1) + (slot & 1);
         sl[0] = rc.x;
         sl[2] = rc.y;
@@ -171,8 +183,24 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
         for (int i = 0; i < n_pairs; ++i) {
             const int k = (head + i) & (SD_RING / 2 - 1);
             const ulonglong2 fa = st2[2 * k];       // {f_a, f_b}, {P_a, P_b}
-            const ulonglong2 fb = st2[2 * k + 1];   // {Pc_a, Pc_b}, {Ps_a, Ps_b}
             const int2 pp = sp2[k];
+            if constexpr (HALF) {
+                // x in FP32, then the window and the reciprocal in packed 16-bit arithmetic;
+                // each product of two 16-bit values, exact in FP32, is added to the window
+                // (of records still scaled by 2^e) with one rounding
+                const uint32_t P2 = (uint32_t)fa.y, Pc2 = (uint32_t)(fa.y >> 32);
+                const uint32_t Ps2 = reinterpret_cast<const uint32_t*>(st2 + 2 * k + 1)[0];
+                float xa, xb;
+                pk_unpack(pk_fma(nsg2, fa.x, xj2), xa, xb);
+                const uint32_t w = fma2<PREC>(C2, Pc2, fma2<PREC>(S2, Ps2, P2));
+                const uint32_t q = rcp2<PREC>(pack2<PREC>(xa, xb));
+                // (one after the other: a lane's sample of the second image is another lane's of
+                // the first)
+                winl[pp.x] = mixed_fma<PREC, false>(winl[pp.x], w, q);
+                winl[pp.y] = mixed_fma<PREC, true>(winl[pp.y], w, q);
+                continue;
+            }
+            const ulonglong2 fb = st2[2 * k + 1];   // {Pc_a, Pc_b}, {Ps_a, Ps_b}
             float va, vb;
             if constexpr (PREC == PREC_FP32) {
                 const unsigned long long x2 = pk_fma(nsg2, fa.x, xj2);
@@ -180,21 +208,6 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
                 float xa, xb;
                 pk_unpack(x2, xa, xb);
                 pk_unpack(pk_mul(w2, pk_pack(ism_rcp(xa), ism_rcp(xb))), va, vb);
-            } else if constexpr (HALF) {
-                // x in FP32, then the window and the reciprocal in packed 16-bit arithmetic;
-                // the products of two 16-bit values are exact in FP32
-                float xa, xb, Pa, Pb, Pca, Pcb, Psa, Psb;
-                pk_unpack(pk_fma(nsg2, fa.x, xj2), xa, xb);
-                pk_unpack(fa.y, Pa, Pb);
-                pk_unpack(fb.x, Pca, Pcb);
-                pk_unpack(fb.y, Psa, Psb);
-                const uint32_t w = fma2<PREC>(C2, pack2<PREC>(Pca, Pcb), fma2<PREC>(S2, pack2<PREC>(Psa, Psb),
-                                                                                   pack2<PREC>(Pa, Pb)));
-                va = 0.0f;
-                vb = 0.0f;
-                mixed_fma2<PREC>(va, vb, w, rcp2<PREC>(pack2<PREC>(xa, xb)));
-                va *= dscale;
-                vb *= dscale;
             } else if constexpr (PREC == PREC_LUT) {
                 float w0a, w0b, w1a, w1b, ra, rb;
                 pk_unpack(fa.x, w0a, w0b);
@@ -274,7 +287,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
             float v = win_all[p];
 #pragma unroll
             for (int w = 1; w < SD_WARPS; ++w) v += win_all[w * winp + p];
-            row[lane] = v;
+            row[lane] = v * dscale;
         }
         {
             float v = 0.0f;
@@ -284,7 +297,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
 #pragma unroll
                 for (int w = 1; w < SD_WARPS; ++w) v += win_all[w * winp + p];
             }
-            row[32 + lane] = v;
+            row[32 + lane] = v * dscale;
         }
     }
 }
