@@ -17,6 +17,15 @@
 // also checks that source and receiver lie strictly inside the room (and that
 // a patterned receiver has a non-zero orientation); a pair that does not gets
 // S = +inf everywhere, i.e. no image survives.
+//
+// Bound: the chain of FP64 instructions of a CTA.  GB300 starts an FP64 warp instruction
+// on a quarter of an SM every ~64 cycles, so each one of a chain costs that much, whether
+// one lane or 32 need it.  Hence a CTA per RIR and axis (a launch of 1 to 50 RIRs leaves
+// most SMs idle), each wall's powers once per CTA instead of two to six per image, the
+// checks in FP32 (exact: the values are FP32) on one warp and f_s / c on another.  Under
+// the profiler, per launch: one RIR 5.6 -> 4.1 us, 128 RIRs 9.5 -> 6.5, 51 rooms with the
+// backward's tables 9.0 -> 5.6, one room of 64 taps with its coefficient tables 8.9 -> 7.7;
+// 512 RIRs of few images per axis, bound by the CTAs' start, 10.3 as before.
 #include <cmath>
 
 #include "ism_device.cuh"
@@ -37,29 +46,38 @@ __device__ double dpow_int(double b, int e)
 // Chebyshev coefficients of 8 of the tap functions g_t(f) = delta'(t - H + 1 - f) (eq. (6))
 // of a window of N_w taps, f = (u + 1) / 2: interpolated at the Chebyshev-Gauss nodes
 // u_k = cos(pi (k + 1/2) / N), c_i = (2 / N) sum_k g_t(u_k) T_i(u_k), c_0 halved, in FP64.
-// (GB300's FP64 pipe is narrow: 8 taps per CTA spread the ~100 values a tap over the SMs
-// beside the geometry CTAs, which take longer.)
+// (8 taps per CTA spread the ~100 values a tap over the SMs; the chain of FP64 instructions
+// is what takes the time, so the cosines of T_i and 1 / N are one warp's work meanwhile.)
 __device__ void cheb_table(const JobDev& J, int N, int tap0, float* tab)
 {
-    __shared__ double gv[8][ISM_CHEB_MAX], cs[ISM_CHEB_MAX][ISM_CHEB_MAX];   // g_t(u_k); T_i(u_k)
-    for (int e = threadIdx.x; e < 8 * N; e += blockDim.x) {
-        const int k = e % N, t = tap0 + e / N;
-        const double f = 0.5 * (cospi((k + 0.5) / N) + 1.0);
-        const int j = t - J.H + 1;
-        const double x = (double)j - f, Nw = (double)J.Nw;
-        double v = 0.0;
-        if (t < 2 * J.H && fabs(x) < 0.5 * Nw)   // sin(pi (j - f)) = (-1)^(j + 1) sin(pi f)
-            v = 0.5 * (1.0 + cospi(2.0 * x / Nw)) * ((j & 1) ? 1.0 : -1.0) * sinpi(f) /
-                (3.141592653589793238462643383279502884 * x);
-        gv[e / N][k] = v;
+    __shared__ double gv[8][ISM_CHEB_MAX], cs[ISM_CHEB_MAX + 1], inv_s;   // g_t(u_k); cos(pi j / 2 N); 1 / N
+    if (threadIdx.x >= 96) {   // the last warp, while the others evaluate the tap functions
+        const int j = threadIdx.x - 96;
+        if (j <= N) cs[j] = cospi(0.5 * j / N);
+        if (j == 0) inv_s = 1.0 / N;
+    } else {
+        for (int e = threadIdx.x; e < 8 * N; e += 96) {
+            const int k = e % N, t = tap0 + e / N;
+            const double f = 0.5 * (cospi((k + 0.5) / N) + 1.0);
+            const int j = t - J.H + 1;
+            const double x = (double)j - f, Nw = (double)J.Nw;
+            double v = 0.0;
+            if (t < 2 * J.H && fabs(x) < 0.5 * Nw)   // sin(pi (j - f)) = (-1)^(j + 1) sin(pi f)
+                v = 0.5 * (1.0 + cospi(2.0 * x / Nw)) * ((j & 1) ? 1.0 : -1.0) * sinpi(f) /
+                    (3.141592653589793238462643383279502884 * x);
+            gv[e / N][k] = v;
+        }
     }
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) cs[e / N][e % N] = cospi((e / N) * (e % N + 0.5) / N);
     __syncthreads();
     for (int e = threadIdx.x; e < 8 * N; e += blockDim.x) {
         const int i = e / 8, t = tap0 + e % 8;
         double c = 0.0;
-        for (int k = 0; k < N; ++k) c += gv[e % 8][k] * cs[i][k];
-        tab[i * 32 * J.slots + t] = (float)(c * (i == 0 ? 1.0 : 2.0) / N);
+        for (int k = 0; k < N; ++k) {   // T_i(u_k) = cos(pi i (2 k + 1) / 2 N), folded into the first quarter
+            int q = i * (2 * k + 1) % (4 * N);
+            q = q > 2 * N ? 4 * N - q : q;
+            c += gv[e % 8][k] * (q > N ? -cs[2 * N - q] : cs[q]);
+        }
+        tab[i * 32 * J.slots + t] = (float)(c * (i == 0 ? inv_s : 2.0 * inv_s));
     }
 }
 
@@ -67,6 +85,7 @@ __global__ void __launch_bounds__(128) geometry_kernel(const __grid_constant__ J
                                                        float4* dtbl, uint32_t* status, float* tabs, int n_rir)
 {
     if ((int)blockIdx.x >= n_rir) {   // the coefficient tables: ISM_CHEB_TAB_CTAS CTAs each
+        if (blockIdx.y > 0) return;
         const int k = ((int)blockIdx.x - n_rir) / ISM_CHEB_TAB_CTAS, c = ((int)blockIdx.x - n_rir) % ISM_CHEB_TAB_CTAS;
         for (int i = 0; i < t.n_jobs; ++i) {
             const JobDev& J = t.j[i];
@@ -77,7 +96,8 @@ __global__ void __launch_bounds__(128) geometry_kernel(const __grid_constant__ J
         }
         return;
     }
-    const long long g = blockIdx.x;  // one CTA per RIR of the launch set
+    const long long g = blockIdx.x;  // one CTA per RIR of the launch set and axis
+    const int a = blockIdx.y;
     const int jid = ism_find_job(t, g, [](const JobDev& j) { return j.rir_base; });
     const JobDev& J = t.j[jid];
     const int r = (int)(g - J.rir_base);
@@ -86,53 +106,63 @@ __global__ void __launch_bounds__(128) geometry_kernel(const __grid_constant__ J
     const float* pr = J.pos_rcv + 3 * i_rcv;
 
     __shared__ int ok_s;
-    __shared__ double ps_s[3], pr_s[3], beta_s[6];
-    if (threadIdx.x == 0) {
-        int ok = 1, ok_beta = 1;
-        for (int w = 0; w < 6; ++w) {
-            const float b = ism_job_beta(J, w);   // checked on the host unless it lives on the device
-            beta_s[w] = (double)b;
-            if (J.beta_dev && !(fabsf(b) <= 1.0f)) ok_beta = 0;
+    __shared__ double k_s, pw[2][32], pw32[2];   // f_s / c; beta_w^0 .. beta_w^31 of the axis's walls, beta_w^32
+    const double xs = (double)ps[a], xr = (double)pr[a];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        double b = (double)ism_job_beta(J, 2 * a + warp), p = 1.0;   // 0^0 = 1: the direct path keeps weight 1
+        for (int i = 0; i < 5 && 4 << i <= J.N[a] + 4; ++i, b *= b)   // (exponents up to N / 4 + 1)
+            if (lane >> i & 1) p *= b;
+        pw[warp][lane] = p;
+        if (lane == 0) pw32[warp] = b;
+    } else if (warp == 2) {   // all in FP32, exactly: the coordinates and coefficients are FP32 values
+        bool in = true, apart = false, dir = false, beta = true;
+        if (lane < 3) {
+            const float s = ps[lane], m = pr[lane];
+            in = s > 0.0f && m > 0.0f && (double)fmaxf(s, m) < J.L[lane];   // (a NaN fails s > 0 or m > 0)
+            apart = s != m;
+            if (J.mic_alpha != 1.0f) {
+                const float o = J.orient_rcv[3 * i_rcv + lane];
+                in = in && fabsf(o) < __int_as_float(0x7f800000);
+                dir = o != 0.0f;
+            } else {
+                dir = true;
+            }
         }
-        if (!ok_beta) atomicOr(status, (uint32_t)ISM_DEVICE_FLAG_BETA);
-        double d2 = 0.0;
-        for (int a = 0; a < 3; ++a) {
-            double xs = ps[a], xr = pr[a];
-            ps_s[a] = xs;
-            pr_s[a] = xr;
-            if (!(xs > 0.0 && xs < J.L[a] && xr > 0.0 && xr < J.L[a])) ok = 0;
-            d2 += (xs - xr) * (xs - xr);
+        if (lane < 6 && J.beta_dev) beta = fabsf(ism_job_beta(J, lane)) <= 1.0f;   // (else checked on the host)
+        const bool ok = __all_sync(~0u, in) && __any_sync(~0u, apart) && __any_sync(~0u, dir);
+        beta = __all_sync(~0u, beta);
+        if (lane == 0) {
+            if (!beta) atomicOr(status, (uint32_t)ISM_DEVICE_FLAG_BETA);
+            if (!ok) atomicOr(status, (uint32_t)ISM_DEVICE_FLAG_POSITION);
+            ok_s = ok && beta;
         }
-        if (!(d2 > 0.0)) ok = 0;
-        if (J.mic_alpha != 1.0f) {
-            const float* o = J.orient_rcv + 3 * i_rcv;
-            const double oo = (double)o[0] * o[0] + (double)o[1] * o[1] + (double)o[2] * o[2];
-            if (!(oo > 0.0) || !(oo < 1e300)) ok = 0;
-        }
-        ok_s = ok && ok_beta;
-        if (!ok) atomicOr(status, (uint32_t)ISM_DEVICE_FLAG_POSITION);
+    } else if (lane == 0) {
+        k_s = (double)J.fs / (double)J.c;
     }
     __syncthreads();
 
+    const auto power = [&](int w, int e) {
+        const double p = pw[w][e & 31];
+        return e < 32 ? p : p * dpow_int(pw32[w], e >> 5);   // (an axis of more than 124 images)
+    };
     const int n_axis = J.N[0] + J.N[1] + J.N[2];
-    const double k = (double)J.fs / (double)J.c;
-    float4* out = tbl + J.tbl_base + (long long)r * n_axis;
-    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) {
-        int a = (e < J.N[0]) ? 0 : ((e < J.N[0] + J.N[1]) ? 1 : 2);
-        int i = e - (a == 0 ? 0 : (a == 1 ? J.N[0] : J.N[0] + J.N[1]));
+    const double k = k_s, L = J.L[a];
+    const long long first = J.tbl_base + (long long)r * n_axis + (a > 0 ? J.N[0] : 0) + (a > 1 ? J.N[1] : 0);
+    for (int i = threadIdx.x; i < J.N[a]; i += blockDim.x) {
         int n = J.nlo[a] + i;
         bool even = (n % 2) == 0;
         // eq. (1): image coordinate minus receiver coordinate
         double m = even ? (double)n : (double)(n + 1);
-        double off = even ? (ps_s[a] - pr_s[a]) : (-ps_s[a] - pr_s[a]);
-        double u = (m * J.L[a] + off) * k;
+        double off = (even ? xs : -xs) - xr;
+        double u = (m * L + off) * k;
         double S = u * u;
         // eq. (4): hits of the near (x0) and far (x1) wall along this axis
         int an = n < 0 ? -n : n;
         int e0 = even ? an / 2 : (n - 1 < 0 ? 1 - n : n - 1) / 2;
         int e1 = even ? an / 2 : (n + 1 < 0 ? -(n + 1) : n + 1) / 2;
-        const double b0 = beta_s[2 * a], b1 = beta_s[2 * a + 1];
-        double F = dpow_int(b0, e0) * dpow_int(b1, e1);
+        const double f0 = power(0, e0), f1 = power(1, e1);
+        double F = f0 * f1;
         float hi = (float)S;
         float lo = (float)(S - (double)hi);
         if (!ok_s) {
@@ -140,12 +170,12 @@ __global__ void __launch_bounds__(128) geometry_kernel(const __grid_constant__ J
             lo = 0.0f;
             F = 0.0;
         }
-        out[e] = make_float4(hi, lo, (float)F, (float)u);
+        tbl[first + i] = make_float4(hi, lo, (float)F, (float)u);
         if (dtbl) {
-            const double d0 = e0 > 0 ? (double)e0 * dpow_int(b0, e0 - 1) * dpow_int(b1, e1) : 0.0;
-            const double d1 = e1 > 0 ? (double)e1 * dpow_int(b0, e0) * dpow_int(b1, e1 - 1) : 0.0;
-            dtbl[J.tbl_base + (long long)r * n_axis + e] = make_float4(
-                (float)(m * J.L[a] + off), ok_s ? (float)d0 : 0.0f, ok_s ? (float)d1 : 0.0f, even ? 1.0f : -1.0f);
+            const double d0 = e0 > 0 ? (double)e0 * power(0, e0 - 1) * f1 : 0.0;
+            const double d1 = e1 > 0 ? (double)e1 * f0 * power(1, e1 - 1) : 0.0;
+            dtbl[first + i] = make_float4((float)(m * L + off), ok_s ? (float)d0 : 0.0f, ok_s ? (float)d1 : 0.0f,
+                                          even ? 1.0f : -1.0f);
         }
     }
 }
@@ -186,7 +216,7 @@ int ism_launch_geometry(const JobTable& t, const WsPlan& p, char* ws, void* stre
 {
     long long n_rir = p.rir_total;
     if (n_rir <= 0) return 0;
-    geometry_kernel<<<(unsigned)(n_rir + ISM_CHEB_TAB_CTAS * p.cheb_tabs), 128, 0, (cudaStream_t)stream>>>(
+    geometry_kernel<<<dim3((unsigned)(n_rir + ISM_CHEB_TAB_CTAS * p.cheb_tabs), 3), 128, 0, (cudaStream_t)stream>>>(
         t, reinterpret_cast<float4*>(ws + p.tbl_off), p.dtbl_off ? reinterpret_cast<float4*>(ws + p.dtbl_off) : nullptr,
         reinterpret_cast<uint32_t*>(ws + p.status_off), reinterpret_cast<float*>(ws + p.lut_off), (int)n_rir);
     return (int)cudaGetLastError();
