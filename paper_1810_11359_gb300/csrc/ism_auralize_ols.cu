@@ -16,8 +16,8 @@
 // registers of one CTA (256 threads x 16 points) and no intermediate goes to
 // device memory: an RIR is read once (its blocks' overlap, Lb / V, from L2).
 // The 48 kHz array (64 segments of 900 samples, 8 microphones, RIRs of 57,600):
-// 4.9 k DFTs of 4096 points instead of 324 of 131,072, 97 us instead of 367.  Its sums
-// (81 us) wait for L2 and shared memory with 16 warps per SM at 44 % of the issue slots;
+// 5.1 k DFTs of 4096 points instead of 324 of 131,072, 94 us instead of 367.  Its sums
+// (80 us) wait for L2 and shared memory with 16 warps per SM at 45 % of the issue slots;
 // samples of the next piece fetched into registers (spills: 112 us) or by cp.async (a second
 // barrier and 32 more shared loads a thread: 105 us) cost more than the waits.
 //
@@ -413,9 +413,11 @@ bool ism_auralize_ols_plan(int n_x, int P, int M, int n_S, bool uniform, int log
     if (!ao_sizes(n_x, P, M, n_S, uniform, pl, &flops)) return false;
     const double N = (double)(1ll << logN);
     if (flops > 1.3 * 5.0 * N * logN * ((double)P * (1.0 + pl.n_pairs) + pl.n_pairs)) return false;
-    // groups of pieces: a few CTAs per SM slot over the launch
+    // groups of pieces: the least that give 1.85 CTAs per slot of the launch (2 per SM); more
+    // only add products to write and sum.  Groups 1 to 5, us: 148 (block, pair)s, 185 121 95
+    // 94 97; 204, 101 73 73 77; 208, 70 64 60 64 66; 246, 92 70 64 68; 32, 178 101 76 64 64
     const long long units = (long long)pl.NB * pl.n_pairs;
-    pl.G = (int)std::max(1LL, std::min(8LL, (8 * 304 + units - 1) / units));
+    pl.G = (int)std::max(1LL, std::min(8LL, (562 + units - 1) / units));
     for (;; --pl.G) {
         size_t off = 0;
         auto take = [&](size_t bytes) {

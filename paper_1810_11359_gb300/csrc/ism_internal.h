@@ -7,15 +7,22 @@
 //   geometry  per RIR and axis: image offsets squared in samples^2 (FP64 ->
 //             float-float) and wall-reflection products (Section 2.1, eq. (1),
 //             eq. (4)); checks the positions.
-//   enum(a)   per RIR and range of grid columns: delays of the images in
-//             reach (eq. (2)-(3)), culling of those whose window misses
-//             [0, n_ism), counts per 32-sample delay bin.
+//   shell     one CTA per (RIR, shell of delay bins): enumerates the shell's images
+//             itself (delays of eq. (2)-(3)) and leaves the bins' window rows, by
+//             Chebyshev moments (FP32, dense bins; a table of coefficients from the
+//             geometry launch unless the window has 32 taps) or tap by tap (32-tap
+//             windows: FP32 with sparse bins, the other tap arithmetics).  A set that
+//             holds both runs them on two streams.
+//   Jobs of neither (other windows: sparse bins, under 16 taps, reduced arithmetics):
+//   enum(a)   per RIR and range of grid columns: delays of the images in reach, culling
+//             of those whose window misses [0, n_ism), counts per 32-sample delay bin.
 //   scan(b)   exclusive prefix over the counts: bin offsets (counting sort).
 //   enum(a')  the same walk, scattering packed image ids into their bins in
 //             a fixed order (stable counting sort).
 //   accum(c)  one CTA per (RIR, ISM_ACC_BPC delay bins), one warp per bin:
 //             the windowed sinc (eq. (6)) of every image of the bin into a
 //             register window, stored as the bin's window row.
+//   Then, for all:
 //   finalize  per RIR: each sample is the sum of the rows of the bins that
 //             cover it, in bin order (eq. (5)); fits the envelope amplitude
 //             of the diffuse tail (Section 2.2).
