@@ -767,15 +767,20 @@ def run_moving_source(args, world, rank, dist, quiet=False):
     peak_tops = n_sm * 128 * sm_mhz * 1e6 / 1e12
     macs = pr.shape[0] * x.numel() * n_s
     rirs = ps.shape[0] * pr.shape[0]
-    # the FFT form's own work: one length-N complex DFT per segment, per point and
-    # microphone pair and per pair's inverse (5 N log2 N flops each, the radix-2
-    # count), and one complex multiply-add (8 flops) per point, pair and bin
+    # the FFT form's own work (overlap-save, 4096-point DFTs, blocks of V outputs): one complex
+    # DFT per segment, per (segment, block that it reaches, microphone pair) and per (block,
+    # pair)'s inverse (5 N log2 N flops each, the radix-2 count), and one complex multiply-add
+    # (8 flops) per segment, block reached, pair and bin
     n_out = x.numel() + n_s - 1
-    logN = max(4, int(math.ceil(math.log2(n_out))))
-    Nf = 1 << logN
+    Nf = 4096
+    seg = -(-x.numel() // ps.shape[0])
+    V = Nf - seg + 1
+    blocks = -(-n_out // V)
     pairs = (pr.shape[0] + 1) // 2
-    n_dft = ps.shape[0] * (1 + pairs) + pairs
-    fft_flops = 5.0 * Nf * logN * n_dft + 8.0 * ps.shape[0] * pairs * Nf
+    starts = [p * x.numel() // ps.shape[0] for p in range(ps.shape[0] + 1)]
+    reached = sum((min(n_out, starts[p + 1] + n_s - 1) - 1) // V - starts[p] // V + 1 for p in range(ps.shape[0]))
+    n_dft = ps.shape[0] + (reached + blocks) * pairs
+    fft_flops = 5.0 * Nf * 12 * n_dft + 8.0 * reached * pairs * Nf
     peak_tflops = 2.0 * peak_tops
     from paper_1810_11359_gb300 import replicas
     ms = replicas.max_over_ranks(ms, device=dev)           # the slowest rank's step (replicas)
@@ -793,7 +798,7 @@ def run_moving_source(args, world, rank, dist, quiet=False):
         "direct_form_ms": direct_ms,
         "fft_speedup_vs_direct": direct_ms / au_ms,
         "fft_vs_direct_max_err_rel_peak": fft_vs_direct,
-        "roofline": {"bound": "alu", "kernel": "af_cols_kernel + af_rows_warp_kernel + af_combine_kernel + af_icols_kernel (FFT form)",
+        "roofline": {"bound": "alu", "kernel": "ao_piece_kernel + ao_sum_kernel + ao_out_kernel (FFT form, overlap-save)",
                      "achieved": fft_flops / (au_ms * 1e-3) / 1e12, "peak": peak_tflops, "unit": "TFLOP/s (FP32)",
                      "frac": fft_flops / (au_ms * 1e-3) / 1e12 / peak_tflops, "flops_per_step": fft_flops,
                      "dft_length": Nf, "dfts_per_step": n_dft,
