@@ -164,6 +164,17 @@ const float* cheb_coefficients(bool forward)
     return forward ? cf : ca;
 }
 
+// Image sources in reach of one RIR of a job: the grid, or the sphere of
+// radius n_ism + H samples (its volume over the room's), whichever is smaller.
+double images_in_reach(const Validated& v)
+{
+    const ism_job& in = v.job;
+    const double k = (double)in.fs / (double)in.room.c;
+    const double reach = ((double)v.n_ism + v.H) / k;
+    const double vol = in.room.L[0] * in.room.L[1] * in.room.L[2];
+    return std::min((double)in.nb_img[0] * in.nb_img[1] * in.nb_img[2], 4.18879020478639 * reach * reach * reach / vol);
+}
+
 // Lays the launch set out in the workspace from byte offset `base` on (the
 // status word is always at offset 0, shared by every launch set of a call).
 // binned: as if FP32 windows of other than 32 taps went through binned image
@@ -419,14 +430,24 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
     p.env_slots = backward ? 0 : vslot;
     p.enum_ctas = ecta;
     p.acc_ctas = acta;
-    // Small launch sets: thinner Chebyshev shells, so that the fused launch still fills
-    // the GPU (ISM_FILL_CTAS CTAs at least; a single RIR would otherwise run on ~20
-    // SMs): from 8 bins down to 1.  The moment sums are exact integers and each bin's
-    // fixed-point scale depends on that bin alone, so a job's result does not depend on
-    // the thickness, nor on the launch set it shares.  (The direct form keeps each job's
-    // own thickness: there the CTA split sets the order of the floating-point sums.)
+    // Small launch sets: thinner Chebyshev shells, from 8 bins down to 1, so that the fused
+    // launch fills the GPU (ISM_FILL_CTAS CTAs at least; a single RIR would otherwise run on
+    // ~20 SMs), and so that a launch of one wave or less whose CTAs hold many images is not
+    // as long as its outermost shells (each shell's images grow as the square of its delay):
+    // twice the CTAs, half as long, the heaviest first.  Accumulation, us, 8 / 4 / 2 bins:
+    // 16 RIRs of 64 taps (704 CTAs, 44,000 images each) 307 / 246 / 295; 8 of 32 taps (304;
+    // 10,800) 63 / 55 / 51; 18 (684) 82 / 73 / 96; 32 (1216) 106 / 120 / 163; 24 (624; 7200)
+    // 61 / 53 / 70; 6 (564; 4300) 57 / 51 / 72; 32 (608; 1700) 31 / 33 / 41: the columns that a
+    // thin shell meets cost as many images' work as it holds.  The moment sums are exact
+    // integers and each bin's fixed-point scale depends on that bin alone, so a job's result
+    // does not depend on the thickness, nor on the launch set it shares.  (The direct form
+    // keeps each job's own thickness: there the CTA split sets the order of the
+    // floating-point sums.)
     t.shell_bins = ISM_SHELL_BINS;
-    if (!backward && scta > 0 && scta < ISM_FILL_CTAS) {
+    if (!backward && scta > 0 && scta <= ISM_WAVE_CTAS) {
+        double images = 0.0;
+        for (int i = 0; i < n; ++i)
+            if (t.j[i].use_cheb) images += (double)t.j[i].n_rir * images_in_reach(vs[i]);
         auto ctas = [&](int bins) {
             long long c = 0;
             for (int i = 0; i < n; ++i)
@@ -434,7 +455,10 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
             return c;
         };
         int bc = ISM_SHELL_BINS;
-        while (bc > 1 && ctas(bc) < ISM_FILL_CTAS) bc >>= 1;
+        for (long long c; bc > 1; bc >>= 1) {
+            c = ctas(bc);
+            if (c >= ISM_FILL_CTAS && (c > ISM_WAVE_CTAS || images < ISM_THIN_IMAGES * (double)c)) break;
+        }
         t.shell_bins = bc;
         scta = 0;
         t.shell_gmax = 0;
@@ -506,17 +530,6 @@ ism_status validate_all(const ism_job* jobs, int n_jobs, std::vector<Validated>&
         }
     }
     return ISM_OK;
-}
-
-// Image sources in reach of one RIR of a job: the grid, or the sphere of
-// radius n_ism + H samples (its volume over the room's), whichever is smaller.
-double images_in_reach(const Validated& v)
-{
-    const ism_job& in = v.job;
-    const double k = (double)in.fs / (double)in.room.c;
-    const double reach = ((double)v.n_ism + v.H) / k;
-    const double vol = in.room.L[0] * in.room.L[1] * in.room.L[2];
-    return std::min((double)in.nb_img[0] * in.nb_img[1] * in.nb_img[2], 4.18879020478639 * reach * reach * reach / vol);
 }
 
 // Execution schedule of a forward call: launch sets (<= ISM_MAX_JOBS jobs

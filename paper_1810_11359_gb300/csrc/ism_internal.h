@@ -63,6 +63,8 @@
 #define ISM_SHELL_BINS 8          // delay bins per CTA of the fused Chebyshev accumulation
 #define ISM_SD_BINS 32            // delay bins per CTA of the fused direct accumulation
 #define ISM_FILL_CTAS 304         // fused CTAs a launch set should have at least (two per SM of a GB300)
+#define ISM_WAVE_CTAS 760         // fused CTAs that run at once (five per SM)
+#define ISM_THIN_IMAGES 3500.0    // images per fused CTA from which thinner shells balance a single wave
 
 // Device-side description of one job.  Everything the kernels need is here
 // so that a whole launch set takes its jobs as one kernel parameter.
