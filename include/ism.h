@@ -523,6 +523,18 @@ typedef enum {
     ISM_AURALIZE_FFT = 2
 } ism_auralize_method;
 
+/* The forms that the methods take. */
+typedef enum {
+    ISM_AURALIZE_FORM_DIRECT = 0,
+    ISM_AURALIZE_FORM_FOUR_STEP = 1,
+    ISM_AURALIZE_FORM_OVERLAP_SAVE = 2
+} ism_auralize_form;
+
+/* The form that ism_auralize_ex takes for these sizes and this method, with
+ * starts given or the uniform cut, and a workspace of
+ * ism_auralize_workspace_size() bytes.  Host only. */
+ism_status ism_auralize_form_of(int n_x, int n_points, int n_mics, int n_S, int method, int given_starts, int* form);
+
 /* Workspace bytes of ism_auralize_ex for this method (0 when it takes the
  * direct form).  Host only. */
 ism_status ism_auralize_workspace_size(int n_x, int n_points, int n_mics, int n_S, int method, size_t* bytes);

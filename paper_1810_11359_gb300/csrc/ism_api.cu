@@ -1601,23 +1601,44 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
     return ISM_OK;
 }
 
-// The automatic choice of ism_auralize_ex, from times estimated at measured rates: the
-// direct form does n_mics n_x n_S multiply-adds (20.5 T/s on the 48 kHz array's
-// filtering); the four-step FFT form about 4 N log2 N lane operations per length-N DFT
-// (one per segment, one per microphone pair and point, one inverse per pair) and 4 per
-// product of spectra (8.0 T/s); the overlap-save form as its estimate says.  64 points x
-// 2 microphones, RIRs of 4800 samples: 129 us direct, 33 us overlap-save.
-static bool auralize_fft_pays(int n_x, int n_points, int n_mics, int n_S)
+// The form that ism_auralize_ex takes (an ism_auralize_form), from the sizes alone, with the
+// plans: *af with the default chunk (of *af_need bytes of workspace), *ao.  -1: the FFT form
+// is asked for an output too long for it.
+// The automatic choice compares times estimated at measured rates.  Four-step against
+// direct: about 4 N log2 N lane operations per length-N DFT (one per segment, one per
+// microphone pair and point, one inverse per pair) and 4 per product of spectra (8.0 T/s)
+// against n_mics n_x n_S multiply-adds (20.5 T/s).  Overlap-save, where its plan exists,
+// as the plan says, against the multiply-adds that the direct kernel issues: microphones
+// padded to 1, 2, 4 or 8 a CTA, a segment's taps to whole chunks of 128 for every tile of
+// 128 outputs (14 to 22 T/s of them; 1 microphone 9 to 14).  Direct and overlap-save, us:
+// 64 points x 2 microphones, RIRs of 4800 samples, 54 and 42; 941 x 8, 4858, segments of
+// 128 samples, 489 and ~310; 100 x 1, 4800, 44 and 47.  892 x 2, whose piece spectra do not
+// fit: 206 direct, 4370 four-step.
+static int auralize_form(int n_x, int n_points, int n_mics, int n_S, bool uniform, int method, AfPlan* af,
+                         size_t* af_need, AoPlan* ao)
 {
-    const long long n_out = (long long)n_x + n_S - 1;
-    int logN = 4;
-    while ((1ll << logN) < n_out) ++logN;
-    if (logN > 20) return false;
-    const double N = (double)(1ll << logN);
-    const double pairs = (double)((n_mics + 1) / 2);
-    const double fft = ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * logN + (double)n_points * pairs * 4.0 * N;
+    if (method == ISM_AURALIZE_DIRECT) return ISM_AURALIZE_FORM_DIRECT;
+    if (ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, 0, af, af_need) != 0)
+        return method == ISM_AURALIZE_FFT ? -1 : (int)ISM_AURALIZE_FORM_DIRECT;
+    // many short segments: overlap-save with one short DFT length, in the least workspace of
+    // the four-step form (one point's chunk and the spectra), so that its choice does not
+    // depend on the workspace's size, nor then the result
+    const size_t seq = (size_t)af->N * 8;
+    const size_t least = (size_t)(1 + af->n_grp) * af->n_pairs * seq + (size_t)(1 + af->n_pairs) * seq;
+    const bool ols = ism_auralize_ols_plan(n_x, n_points, n_mics, n_S, uniform, af->logN, least, ao);
+    const int fft_form = ols ? ISM_AURALIZE_FORM_OVERLAP_SAVE : ISM_AURALIZE_FORM_FOUR_STEP;
+    if (method == ISM_AURALIZE_FFT) return fft_form;
+    const double N = (double)af->N, pairs = (double)af->n_pairs;
+    const double fft =
+        ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * af->logN + (double)n_points * pairs * 4.0 * N;
     const double direct = (double)n_mics * (double)n_x * (double)n_S;
-    return direct > 2.55 * fft || 1.0e-5 + direct / 2.05e13 > ism_auralize_ols_seconds(n_x, n_points, n_mics, n_S);
+    if (direct > 2.55 * fft) return fft_form;
+    const double len = (double)n_x / n_points;
+    const double padded = std::ceil((len + 127.0) / 128.0) * 128.0 / len;
+    const int mics = n_mics <= 2 ? n_mics : n_mics <= 4 ? 4 : (n_mics + 7) / 8 * 8;
+    const double issued = (double)mics * (double)n_x * (double)n_S * padded;
+    return ols && 1.0e-5 + issued / (mics == 1 ? 1.4e13 : 2.05e13) > ao->seconds ? ISM_AURALIZE_FORM_OVERLAP_SAVE
+                                                                                 : ISM_AURALIZE_FORM_DIRECT;
 }
 
 static ism_status auralize_args(const float* signal, int n_x, const float* rirs, int n_points, int n_mics, int n_S,
@@ -1632,24 +1653,50 @@ static ism_status auralize_args(const float* signal, int n_x, const float* rirs,
     return ISM_OK;
 }
 
+static ism_status auralize_sizes(int n_x, int n_points, int n_mics, int n_S, int method)
+{
+    if (n_x < 1 || n_points < 1 || n_mics < 1 || n_S < 1)
+        return fail(ISM_ERR_INVALID_ARG, "need n_x, n_points, n_mics, n_S >= 1");
+    if (method < ISM_AURALIZE_AUTO || method > ISM_AURALIZE_FFT)
+        return fail(ISM_ERR_INVALID_ARG, "method = %d is not an ism_auralize_method", method);
+    return ISM_OK;
+}
+
+static ism_status auralize_too_long(int n_x, int n_S)
+{
+    return fail(ISM_ERR_UNSUPPORTED, "output of %lld samples exceeds the FFT form's 2^20", (long long)n_x + n_S - 1);
+}
+
+ism_status ism_auralize_form_of(int n_x, int n_points, int n_mics, int n_S, int method, int given_starts, int* form)
+{
+    g_last_error.clear();
+    if (!form) return fail(ISM_ERR_INVALID_ARG, "form must not be NULL");
+    ism_status st = auralize_sizes(n_x, n_points, n_mics, n_S, method);
+    if (st != ISM_OK) return st;
+    AfPlan af;
+    AoPlan ao;
+    size_t need = 0;
+    const int f = auralize_form(n_x, n_points, n_mics, n_S, !given_starts, method, &af, &need, &ao);
+    if (f < 0) return auralize_too_long(n_x, n_S);
+    *form = f;
+    return ISM_OK;
+}
+
 ism_status ism_auralize_workspace_size(int n_x, int n_points, int n_mics, int n_S, int method, size_t* bytes)
 {
     g_last_error.clear();
     if (!bytes) return fail(ISM_ERR_INVALID_ARG, "bytes must not be NULL");
     *bytes = 0;
-    if (n_x < 1 || n_points < 1 || n_mics < 1 || n_S < 1)
-        return fail(ISM_ERR_INVALID_ARG, "need n_x, n_points, n_mics, n_S >= 1");
-    if (method < ISM_AURALIZE_AUTO || method > ISM_AURALIZE_FFT)
-        return fail(ISM_ERR_INVALID_ARG, "method = %d is not an ism_auralize_method", method);
-    const bool fft = method == ISM_AURALIZE_FFT ||
-                     (method == ISM_AURALIZE_AUTO && auralize_fft_pays(n_x, n_points, n_mics, n_S));
-    if (!fft) return ISM_OK;
-    AfPlan pl;
-    size_t need = 0;
-    if (ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, 0, &pl, &need))
-        return fail(ISM_ERR_UNSUPPORTED, "output of %lld samples exceeds the FFT form's 2^20",
-                    (long long)n_x + n_S - 1);
-    *bytes = need;
+    ism_status st = auralize_sizes(n_x, n_points, n_mics, n_S, method);
+    if (st != ISM_OK) return st;
+    for (const bool uniform : {true, false}) {   // (the starts come with the call)
+        AfPlan af;
+        AoPlan ao;
+        size_t need = 0;
+        const int form = auralize_form(n_x, n_points, n_mics, n_S, uniform, method, &af, &need, &ao);
+        if (form < 0) return auralize_too_long(n_x, n_S);
+        if (form != ISM_AURALIZE_FORM_DIRECT) *bytes = std::max(*bytes, need);
+    }
     return ISM_OK;
 }
 
@@ -1659,29 +1706,22 @@ ism_status ism_auralize_ex(const float* signal, int n_x, const float* rirs, int 
     g_last_error.clear();
     ism_status st = auralize_args(signal, n_x, rirs, n_points, n_mics, n_S, out);
     if (st != ISM_OK) return st;
-    if (method < ISM_AURALIZE_AUTO || method > ISM_AURALIZE_FFT)
-        return fail(ISM_ERR_INVALID_ARG, "method = %d is not an ism_auralize_method", method);
-    bool fft = method == ISM_AURALIZE_FFT;
+    if ((st = auralize_sizes(n_x, n_points, n_mics, n_S, method)) != ISM_OK) return st;
     AfPlan pl;
+    AoPlan ol;
     size_t need = 0;
-    if (method == ISM_AURALIZE_AUTO && auralize_fft_pays(n_x, n_points, n_mics, n_S) && workspace &&
-        ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need) == 0)
-        fft = true;
-    if (fft) {
+    int form = auralize_form(n_x, n_points, n_mics, n_S, starts == nullptr, method, &pl, &need, &ol);
+    if (method == ISM_AURALIZE_AUTO && form != ISM_AURALIZE_FORM_DIRECT &&
+        (!workspace || ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need) != 0))
+        form = ISM_AURALIZE_FORM_DIRECT;
+    if (form != ISM_AURALIZE_FORM_DIRECT) {
         if (!workspace) return fail(ISM_ERR_INVALID_ARG, "the FFT form needs a workspace");
         if (((uintptr_t)workspace & 255u) != 0) return fail(ISM_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
         const int r = ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need);
-        if (r == -1)
-            return fail(ISM_ERR_UNSUPPORTED, "output of %lld samples exceeds the FFT form's 2^20",
-                        (long long)n_x + n_S - 1);
+        if (r == -1) return auralize_too_long(n_x, n_S);
         if (r == -2)
             return fail(ISM_ERR_WORKSPACE_TOO_SMALL, "workspace of %zu bytes holds no chunk of the FFT form", ws_bytes);
-        // many short segments: overlap-save with one short DFT length (its choice does not
-        // depend on the workspace's size, nor then the result)
-        AoPlan ol;
-        const size_t seq = (size_t)pl.N * 8;   // one point's chunk and the spectra: the least workspace
-        const size_t least = (size_t)(1 + pl.n_grp) * pl.n_pairs * seq + (size_t)(1 + pl.n_pairs) * seq;
-        int e = ism_auralize_ols_plan(n_x, n_points, n_mics, n_S, starts == nullptr, pl.logN, least, &ol)
+        int e = form == ISM_AURALIZE_FORM_OVERLAP_SAVE
                     ? ism_launch_auralize_ols(signal, rirs, starts, out, ol, static_cast<char*>(workspace), stream)
                     : ism_launch_auralize_fft(signal, rirs, starts, out, pl, static_cast<char*>(workspace), stream);
         if (e) return cuda_fail(e, "auralization (FFT) kernels");

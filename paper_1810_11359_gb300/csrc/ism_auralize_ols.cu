@@ -22,7 +22,8 @@
 // barrier and 32 more shared loads a thread: 105 us) cost more than the waits.
 //
 // Two microphones share a complex sequence, as in the four-step form.  Segments
-// longer than Lb are cut into pieces; piece j of segment p has the slot
+// longer than Lb are cut into pieces.  A uniform cut's segments have equally many
+// (cuts: slot cuts p + j); with given starts piece j of segment p has the slot
 // p + floor(a_p / Lb) + j, which no other piece has (starts are non-decreasing),
 // so the slots need no prefix sum over the points.  A CTA takes the pieces of
 // one group (of every G-th that reach its block) and leaves their summed
@@ -186,14 +187,16 @@ __global__ void __launch_bounds__(AO_T) ao_piece_kernel(AoPlan pl, const float* 
     float2* t2 = t1 + AO_N;
     const int c = blockIdx.x;
     ao_tables(t1, t2, nullptr);
-    int lo = 0, hi = pl.P - 1;   // the last point whose first slot is <= c
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (mid + ao_start(mid, pl.n_x, pl.P, starts) / pl.Lb <= c) lo = mid;
-        else hi = mid - 1;
-    }
+    int lo = 0, hi = pl.P - 1;
+    if (pl.cuts) lo = c / pl.cuts;
+    else
+        while (lo < hi) {   // the last point whose first slot is <= c
+            const int mid = (lo + hi + 1) >> 1;
+            if (mid + ao_start(mid, pl.n_x, pl.P, starts) / pl.Lb <= c) lo = mid;
+            else hi = mid - 1;
+        }
     const int a = ao_start(lo, pl.n_x, pl.P, starts), b = ao_start(lo + 1, pl.n_x, pl.P, starts);
-    const long long s0 = (long long)a + (long long)(c - lo - a / pl.Lb) * pl.Lb;
+    const long long s0 = (long long)a + (long long)(c - (pl.cuts ? lo * pl.cuts : lo + a / pl.Lb)) * pl.Lb;
     const int len = s0 >= a && s0 < b ? (int)min((long long)pl.Lb, b - s0) : 0;
     if (threadIdx.x == 0) desc[c] = make_int4(lo, (int)min(s0, (long long)pl.n_x), len, 0);
     __syncthreads();
@@ -382,20 +385,12 @@ static bool ao_sizes(int n_x, int P, int M, int n_S, bool uniform, AoPlan& pl, d
     pl.Lb = uniform ? (seg + cuts - 1) / cuts : std::min(cap, 2 * seg);
     pl.V = AO_N - pl.Lb + 1;
     pl.NB = (pl.n_out + pl.V - 1) / pl.V;
-    const long long slots = (long long)P + n_x / pl.Lb + 1;
+    pl.cuts = uniform ? (seg + pl.Lb - 1) / pl.Lb : 0;
+    const long long slots = uniform ? (long long)P * pl.cuts : (long long)P + n_x / pl.Lb + 1;
     if (slots > 65535 || (long long)pl.NB * 8 * pl.n_pairs > 0x7FFFFFFFll || pl.n_pairs > 65535) return false;
     pl.slots = (int)slots;
-    *flops = ao_flops(pl, uniform ? (double)P * ((seg + pl.Lb - 1) / pl.Lb) : 1.3 * P);
+    *flops = ao_flops(pl, uniform ? (double)P * pl.cuts : 1.3 * P);
     return true;
-}
-
-// Seconds that the form takes, roughly (the array's 1.27 G operations take 97 us; a small
-// filtering's three launches 20 us): for the choice between it and the direct form.
-double ism_auralize_ols_seconds(int n_x, int P, int M, int n_S)
-{
-    AoPlan pl;
-    double flops = 0.0;
-    return ao_sizes(n_x, P, M, n_S, true, pl, &flops) ? 2.0e-5 + flops / 1.2e13 : 1.0e9;
 }
 
 // Whether the overlap-save form takes a filtering, and its plan.  It does where its DFTs'
@@ -406,6 +401,9 @@ double ism_auralize_ols_seconds(int n_x, int P, int M, int n_S)
 // 69; 3.4 (4 points) 73 and 53.
 // ws_min: the workspace that the four-step form needs at least (every workspace that
 // the caller may pass holds that; this form takes no more).
+// out->seconds: the time that the form takes, roughly (the array's 1.27 G operations take
+// 97 us; a small filtering's three launches 25 us), for the choice between it and the
+// direct form; out->total: the workspace it takes.
 bool ism_auralize_ols_plan(int n_x, int P, int M, int n_S, bool uniform, int logN, size_t ws_min, AoPlan* out)
 {
     AoPlan pl;
@@ -429,9 +427,11 @@ bool ism_auralize_ols_plan(int n_x, int P, int M, int n_S, bool uniform, int log
         pl.t1_off = take((size_t)AO_N * sizeof(float2));
         pl.x_off = take((size_t)pl.slots * AO_XN * sizeof(float2));
         pl.y_off = take((size_t)units * pl.G * AO_N * sizeof(float2));
+        pl.total = off;
         if (off <= ws_min) break;
         if (pl.G == 1) return false;
     }
+    pl.seconds = 2.5e-5 + flops / 1.2e13;
     *out = pl;
     return true;
 }

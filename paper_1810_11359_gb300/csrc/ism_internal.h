@@ -239,9 +239,12 @@ struct AoPlan {
     int Lb;      // samples of a piece of a segment, at most
     int V;       // outputs per block: 4096 - Lb + 1
     int NB;      // blocks
-    int slots;   // pieces, with gaps
+    int cuts;    // pieces per segment of a uniform cut; 0: given starts
+    int slots;   // pieces, with gaps where starts are given
     int G;       // groups of pieces per block (their sums are added in group order)
     size_t desc_off, t1_off, x_off, y_off;   // in the workspace
+    size_t total;     // bytes of it
+    double seconds;   // estimated
 };
 
 // Sets the calling thread's ism_last_error_message() and returns s.
@@ -273,7 +276,6 @@ int ism_launch_auralize(const float* x, int n_x, const float* h, int n_points, i
 int ism_auralize_fft_plan(int n_x, int n_points, int n_mics, int n_S, size_t ws_bytes, AfPlan* out, size_t* need);
 int ism_launch_auralize_fft(const float* x, const float* h, const int* starts, float* y, const AfPlan& pl, char* ws,
                             void* stream);
-double ism_auralize_ols_seconds(int n_x, int n_points, int n_mics, int n_S);
 bool ism_auralize_ols_plan(int n_x, int n_points, int n_mics, int n_S, bool uniform, int logN, size_t ws_min,
                            AoPlan* out);
 int ism_launch_auralize_ols(const float* x, const float* h, const int* starts, float* y, const AoPlan& pl, char* ws,

@@ -127,6 +127,7 @@ _SIGS = {
                                          ctypes.c_void_p, ctypes.c_void_p]),
     "ism_auralize": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_int,
                                     ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
+    "ism_auralize_form_of": (ctypes.c_int, [ctypes.c_int] * 6 + [ctypes.POINTER(ctypes.c_int)]),
     "ism_auralize_workspace_size": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                    ctypes.c_int, _P(ctypes.c_size_t)]),
     "ism_auralize_ex": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_int,
@@ -584,6 +585,7 @@ def ism_simulate_backward(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, grad_out,
 
 
 AURALIZE_METHODS = {"auto": 0, "direct": 1, "fft": 2}
+AURALIZE_FORMS = {0: "direct", 1: "four_step", 2: "overlap_save"}
 
 
 def ism_auralize_workspace_size(n_x: int, n_points: int, n_mics: int, n_s: int, method: str = "auto") -> int:
@@ -591,6 +593,14 @@ def ism_auralize_workspace_size(n_x: int, n_points: int, n_mics: int, n_s: int, 
     _check(load().ism_auralize_workspace_size(int(n_x), int(n_points), int(n_mics), int(n_s),
                                               AURALIZE_METHODS[method], ctypes.byref(b)))
     return int(b.value)
+
+
+def ism_auralize_form(n_x: int, n_points: int, n_mics: int, n_s: int, method: str = "auto", given_starts: bool = False) -> str:
+    """The form that ism_auralize takes for these sizes (an AURALIZE_FORMS name)."""
+    f = ctypes.c_int()
+    _check(load().ism_auralize_form_of(int(n_x), int(n_points), int(n_mics), int(n_s), AURALIZE_METHODS[method],
+                                       int(bool(given_starts)), ctypes.byref(f)))
+    return AURALIZE_FORMS[f.value]
 
 
 def ism_auralize(signal, rirs, starts=None, out=None, stream=None, method: Optional[str] = None,
