@@ -511,7 +511,9 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
  * all outputs.  ISM_AURALIZE_DIRECT is ism_auralize (no workspace).
  * ISM_AURALIZE_AUTO takes the FFT form when it is estimated to be faster than
  * the direct form (n_mics n_x n_S multiply-adds; rates measured on GB300) and
- * the workspace holds at least one chunk, else the direct form.
+ * the workspace holds what that form takes (overlap-save: its piece spectra and
+ * block sums, ism_auralize_workspace_size(); four-step: at least one chunk), else
+ * the direct form.
  *   workspace  device, 256-byte aligned, >= ism_auralize_workspace_size()
  *              bytes for the FFT form (scratch; may be NULL for DIRECT);
  *              a larger workspace processes more points per chunk.
@@ -535,8 +537,8 @@ typedef enum {
  * ism_auralize_workspace_size() bytes.  Host only. */
 ism_status ism_auralize_form_of(int n_x, int n_points, int n_mics, int n_S, int method, int given_starts, int* form);
 
-/* Workspace bytes of ism_auralize_ex for this method (0 when it takes the
- * direct form).  Host only. */
+/* Workspace bytes of ism_auralize_ex for this method, with starts given or not
+ * (0 when it takes the direct form either way).  Host only. */
 ism_status ism_auralize_workspace_size(int n_x, int n_points, int n_mics, int n_S, int method, size_t* bytes);
 
 ism_status ism_auralize_ex(const float* signal, int n_x, const float* rirs, int n_points, int n_mics, int n_S,

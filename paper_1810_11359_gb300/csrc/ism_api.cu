@@ -1612,7 +1612,7 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
 // padded to 1, 2, 4 or 8 a CTA, a segment's taps to whole chunks of 128 for every tile of
 // 128 outputs (14 to 22 T/s of them; 1 microphone 9 to 14).  Direct and overlap-save, us:
 // 64 points x 2 microphones, RIRs of 4800 samples, 54 and 42; 941 x 8, 4858, segments of
-// 128 samples, 489 and ~310; 100 x 1, 4800, 44 and 47.  892 x 2, whose piece spectra do not
+// 128 samples, 489 and 205; 100 x 1, 4800, 45 and 43.  892 x 2, whose piece spectra do not
 // fit: 206 direct, 4370 four-step.
 static int auralize_form(int n_x, int n_points, int n_mics, int n_S, bool uniform, int method, AfPlan* af,
                          size_t* af_need, AoPlan* ao)
@@ -1695,6 +1695,8 @@ ism_status ism_auralize_workspace_size(int n_x, int n_points, int n_mics, int n_
         size_t need = 0;
         const int form = auralize_form(n_x, n_points, n_mics, n_S, uniform, method, &af, &need, &ao);
         if (form < 0) return auralize_too_long(n_x, n_S);
+        // (the FFT method keeps the four-step form's, whose least it accepts for either form)
+        if (form == ISM_AURALIZE_FORM_OVERLAP_SAVE && method == ISM_AURALIZE_AUTO) need = ao.total;
         if (form != ISM_AURALIZE_FORM_DIRECT) *bytes = std::max(*bytes, need);
     }
     return ISM_OK;
@@ -1711,14 +1713,16 @@ ism_status ism_auralize_ex(const float* signal, int n_x, const float* rirs, int 
     AoPlan ol;
     size_t need = 0;
     int form = auralize_form(n_x, n_points, n_mics, n_S, starts == nullptr, method, &pl, &need, &ol);
-    if (method == ISM_AURALIZE_AUTO && form != ISM_AURALIZE_FORM_DIRECT &&
-        (!workspace || ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need) != 0))
-        form = ISM_AURALIZE_FORM_DIRECT;
+    // the automatic choice runs in what its form takes, or else directly
+    const bool own = method == ISM_AURALIZE_AUTO && form == ISM_AURALIZE_FORM_OVERLAP_SAVE;
+    int r = 0;
+    if (form >= 0 && form != ISM_AURALIZE_FORM_DIRECT)
+        r = own ? (ws_bytes < ol.total ? -2 : 0) : ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need);
+    if (method == ISM_AURALIZE_AUTO && (!workspace || r != 0)) form = ISM_AURALIZE_FORM_DIRECT;
     if (form != ISM_AURALIZE_FORM_DIRECT) {
         if (!workspace) return fail(ISM_ERR_INVALID_ARG, "the FFT form needs a workspace");
         if (((uintptr_t)workspace & 255u) != 0) return fail(ISM_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
-        const int r = ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need);
-        if (r == -1) return auralize_too_long(n_x, n_S);
+        if (form < 0) return auralize_too_long(n_x, n_S);
         if (r == -2)
             return fail(ISM_ERR_WORKSPACE_TOO_SMALL, "workspace of %zu bytes holds no chunk of the FFT form", ws_bytes);
         int e = form == ISM_AURALIZE_FORM_OVERLAP_SAVE

@@ -5,6 +5,8 @@ The automatic choice has to go by the form that will run: sizes whose piece spec
 the overlap-save form's workspace would otherwise run the four-step form, which its estimate
 never saw (892 points x 2 microphones: 4370 us against 206 us direct).
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -58,6 +60,19 @@ def test_automatic_choice_never_takes_the_four_step_form_for_overlap_saves_time(
             assert M * n_x * n_s > 2.55 * ops, (n_x, P, M, n_s, given)
 
 
+@pytest.mark.parametrize("size", [(57600, 64, 8, 57600), (57600, 64, 2, 4800), (30000, 64, 4, 3200), (144000, 500, 2, 19200)])
+def test_workspace_of_the_overlap_save_form(size):
+    """The automatic choice asks for the overlap-save form's piece spectra (18 KB each; of given
+    starts up to 1.5 a point) and block sums (32 KB each; groups up to 562 CTAs more than the
+    blocks of 2049 outputs or more), not for the four-step form's 64 to 96 MB of chunk."""
+    n_x, P, M, n_s = size
+    pieces = 1.5 * P + n_x / 2048 + 2
+    sums = 562 + ((n_x + n_s - 1) // 2049 + 1) * ((M + 1) // 2)
+    b = ism.ism_auralize_workspace_size(*size, "auto")
+    assert 0 < b <= pieces * (18432 + 16) + sums * 32768 + 32768 + 1024
+    assert b < ism.ism_auralize_workspace_size(*size, "fft") / 2
+
+
 def test_form_arguments():
     with pytest.raises(ism.IsmError):
         ism.ism_auralize_form(0, 1, 1, 1)
@@ -95,3 +110,21 @@ def test_automatic_call_runs_the_chosen_form(n_x, n_points, n_mics, n_s):
         form = ism.ism_auralize_form(n_x, n_points, n_mics, n_s, given_starts=s is not None)
         want = ism.ism_auralize(x, h, starts=s, method="direct" if form == "direct" else "fft")
         assert torch.equal(ism.ism_auralize(x, h, starts=s, method="auto"), want)
+
+
+@pytest.mark.gpu
+def test_automatic_call_with_less_workspace_runs_directly():
+    """One byte below the least that any form takes, and none: the direct form."""
+    torch.cuda.set_device(0)
+    n_x, P, M, n_s = 57600, 64, 2, 4800
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(n_x, generator=g, device="cuda")
+    h = torch.randn((P, M, n_s), generator=g, device="cuda")
+    direct = ism.ism_auralize(x, h, method="direct")
+    out = torch.empty_like(direct)
+    ws = torch.empty(1 << 23, dtype=torch.uint8, device="cuda")
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    for w, n in ((ws, 1 << 20), (None, 0)):
+        ism._check(ism.load().ism_auralize_ex(ptr(x), n_x, ptr(h), P, M, n_s, None, ptr(out), ism.AURALIZE_METHODS["auto"],
+                                              None if w is None else ptr(w), n, ism._stream_ptr(None)))
+        assert torch.equal(out, direct)
