@@ -1717,7 +1717,8 @@ ism_status ism_auralize_ex(const float* signal, int n_x, const float* rirs, int 
     const bool own = method == ISM_AURALIZE_AUTO && form == ISM_AURALIZE_FORM_OVERLAP_SAVE;
     int r = 0;
     if (form >= 0 && form != ISM_AURALIZE_FORM_DIRECT)
-        r = own ? (ws_bytes < ol.total ? -2 : 0) : ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, ws_bytes, &pl, &need);
+        r = own ? (ws_bytes < ol.total ? -2 : 0)   // (no bytes: to the plan, the default size)
+                : ism_auralize_fft_plan(n_x, n_points, n_mics, n_S, std::max<size_t>(ws_bytes, 1), &pl, &need);
     if (method == ISM_AURALIZE_AUTO && (!workspace || r != 0)) form = ISM_AURALIZE_FORM_DIRECT;
     if (form != ISM_AURALIZE_FORM_DIRECT) {
         if (!workspace) return fail(ISM_ERR_INVALID_ARG, "the FFT form needs a workspace");

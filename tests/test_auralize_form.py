@@ -128,3 +128,15 @@ def test_automatic_call_with_less_workspace_runs_directly():
         ism._check(ism.load().ism_auralize_ex(ptr(x), n_x, ptr(h), P, M, n_s, None, ptr(out), ism.AURALIZE_METHODS["auto"],
                                               None if w is None else ptr(w), n, ism._stream_ptr(None)))
         assert torch.equal(out, direct)
+
+
+@pytest.mark.gpu
+def test_fft_method_refuses_a_workspace_of_no_bytes():
+    torch.cuda.set_device(0)
+    x, h, out = torch.ones(3000, device="cuda"), torch.ones((3, 2, 900), device="cuda"), torch.empty((2, 3899), device="cuda")
+    ws = torch.empty(1 << 23, dtype=torch.uint8, device="cuda")   # (so that even an accepting call stays inside)
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    for n_mics in (1, 2):
+        st = ism.load().ism_auralize_ex(ptr(x), 3000, ptr(h), 3, n_mics, 900, None, ptr(out), ism.AURALIZE_METHODS["fft"], ptr(ws),
+                                        0, ism._stream_ptr(None))
+        assert st == 3   # ISM_ERR_WORKSPACE_TOO_SMALL
