@@ -1,7 +1,7 @@
 // ism_accum_cheb.cu -- FP32 accumulation of eq. (5) through a Chebyshev
 // expansion of the windowed sinc in the fractional delay, fused with the
 // enumeration of the images (Section 2.1) it accumulates: 32-tap windows with
-// 8 terms (the text below), other windows of 16 taps or more with 10.
+// 8 terms (the text below), other windows whose taps a series follows with 10.
 //
 // For tap j of an image with delay s = b + f (b integer, f in [0, 1)), the
 // sample b + j receives A delta'(j - f) (eq. (6)).  For a window of exactly
@@ -61,8 +61,9 @@
 // Other windows (the default, 4 ms, is 64 taps at 16 kHz and 176.4 at 44.1 kHz).
 // A window whose end falls inside a sample interval cuts its last taps with a
 // mask, which no polynomial follows, but the window has a double zero there:
-// for 16 taps or more the kink is below 2.7e-8 of the amplitude and degree 9
-// reproduces every tap to that (2.5e-9 without a mask).  The 2 H coefficients
+// the kink falls with the cube of the window's length, and degree 9 reproduces the
+// taps to 2.6e-8 of the amplitude (1e-8 without a mask; norms over the taps) for the
+// windows that this form takes (series_follows_window).  The 2 H coefficients
 // of each term come from a table in the workspace that the geometry launch
 // fills (cheb_table), and the expansion takes 32 taps at a time, each turn's
 // upper half carried into the next.  The terms are converted to integers

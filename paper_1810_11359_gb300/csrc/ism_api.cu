@@ -175,6 +175,21 @@ double images_in_reach(const Validated& v)
     return std::min((double)in.nb_img[0] * in.nb_img[1] * in.nb_img[2], 4.18879020478639 * reach * reach * reach / vol);
 }
 
+// Whether a Chebyshev series keeps the accuracy of the tap functions of the
+// job's window (other than 32 taps).  A window that ends inside a sample interval, theta of
+// it, cuts its outermost taps there; what the series of degree 9 misses of them is at most
+// 0.018 sin(pi theta) / N_w^3 of an image's amplitude (norm over the taps; every N_w from 16 to
+// 256 in steps of 0.1), where the FP32 rounding of a tap-by-tap sum leaves about 1.1e-7.  The
+// rule admits 2.6e-8 of it: windows that end on a sample, any from 80 taps on, and those
+// between that end close to a sample (44.1 taps).  Relative error of RIRs of 17.5,
+// 20.8, 24.8 and 33.3 taps: 3.2, 3.7, 2.4 and 1.4e-7 through the series, 1.0 to 1.1e-7 tap by
+// tap, the form that they take.
+bool series_follows_window(const Validated& v)
+{
+    const double theta = 0.5 * v.Nw - (v.H - 1);   // in (0, 1]
+    return v.Nw >= ISM_CHEB_MIN_NW && v.Nw * v.Nw * v.Nw >= 5.0e5 * std::sin(M_PI * theta);
+}
+
 // Lays the launch set out in the workspace from byte offset `base` on (the
 // status word is always at offset 0, shared by every launch set of a call).
 // binned: as if FP32 windows of other than 32 taps went through binned image
@@ -301,17 +316,16 @@ ism_status plan(const Validated* vs, int n, ism_precision prec, bool backward, J
             const double in_reach = std::min((double)in.nb_img[0] * in.nb_img[1] * in.nb_img[2],
                                              4.18879020478639 * reach * reach * reach / vol);
             const double per_bin = in_reach / (double)((v.n_ism + v.H) / ISM_SB + 1);
-            // Other windows take them from 20 images per bin on, at degree 9, whose series keeps
-            // the per-tap sum's accuracy for every window of ISM_CHEB_MIN_NW taps or more: the
-            // form they take below that has passes over the images to count, scan and scatter
-            // before it.  Measured against it (a call, us): 16 RIRs of 64 taps, 5500 per bin,
+            // Other windows take them from 20 images per bin on, at degree 9, where the series
+            // keeps the per-tap sum's accuracy (series_follows_window): the form they take
+            // otherwise has passes over the images to count, scan and scatter before it.  Measured against it (a call, us): 16 RIRs of 64 taps, 5500 per bin,
             // 2000 -> 350; of 176 taps, 27 per bin, 15 RIRs 63 -> 42 and 512 RIRs 450 -> 415;
             // 6 per bin, 512 RIRs 122 -> 151; of 40 taps, 43 per bin, 512 RIRs 445 -> 329; 11
             // per bin, 131 -> 133.
             const bool taps32 = v.Nw == 32.0;
             J.use_cheb = 0;
             if (prec == ISM_PREC_FP32 && !backward && taps32 && per_bin >= 64.0) J.use_cheb = ISM_CHEB_NF;
-            if (prec == ISM_PREC_FP32 && !backward && !taps32 && per_bin >= 20.0 && v.Nw >= ISM_CHEB_MIN_NW && !binned)
+            if (prec == ISM_PREC_FP32 && !backward && !taps32 && per_bin >= 20.0 && series_follows_window(v) && !binned)
                 J.use_cheb = ISM_CHEB_NW;
             // sparse bins: sorting by offset and padding each offset to a group of 4
             // images costs more than adding every image's taps on its own

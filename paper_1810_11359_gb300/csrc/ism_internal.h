@@ -54,7 +54,7 @@
 #define ISM_CHEB_N 9              // Chebyshev terms of a tap function in the adjoint (degree 8); table stride
 #define ISM_CHEB_NF 8             // Chebyshev terms of the forward's moments (degree 7)
 #define ISM_CHEB_NW 10            // the same for windows other than 32 taps (degree 9)
-#define ISM_CHEB_MIN_NW 16        // shortest window whose taps the series reproduces (see ism_accum_cheb.cu)
+#define ISM_CHEB_MIN_NW 16        // shortest window whose taps a series reproduces (see series_follows_window)
 #define ISM_CHEB_AW 11            // terms of the adjoint for windows other than 32 taps (degree 10)
 #define ISM_CHEB_MAX 12           // terms of any of them, at most
 #define ISM_ADJ_MIN_NW 80         // windows that end inside a sample interval: shortest for the fused adjoint
