@@ -95,7 +95,7 @@ __device__ __forceinline__ float shell_scale(float a_max, float n, float term_ma
     return __int_as_float((e + 127) << 23);
 }
 
-template <int NM>
+template <int NM, bool SPLIT>
 __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_constant__ JobTable t,
                                                                   const float4* __restrict__ tbl,
                                                                   const float* __restrict__ tabs,
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     int jid, r, grp;
     if (!shell_cta(t, blockIdx.x, &jid, &r, &grp)) return;   // CTA-uniform
     const JobDev& J = t.j[jid];
-    if (J.use_cheb != NM) return;   // another instantiation's job
+    if (J.use_cheb != NM || shell_split(J) != SPLIT) return;   // another instantiation's job
     const int B = t.shell_bins;   // bins of this launch's shells: SH_B, fewer for small launch sets
     const int q0 = grp * B;
     const int nb = min(B, J.Q - q0);
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
 
     const float s2_magic = shell_s2_magic(J);
     const float4* Tg = tbl + J.tbl_base + (long long)r * n_axis;
-    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) shell_stage<true>(T, e, Tg[e], s2_magic);
+    for (int e = threadIdx.x; e < n_axis; e += blockDim.x) shell_stage<SPLIT>(T, e, Tg[e], s2_magic);
     if (threadIdx.x == 0) *redo = 0;
     __syncthreads();
 
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     for (int e = threadIdx.x; e < (NM + 1) * SH_RS / 4; e += blockDim.x)
         reinterpret_cast<uint4*>(S)[e] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    shell_walk<SH_WARPS>(sh, T, rowpre, rowy0, n_cols, J.amp_scale, Wf, Wi, Wm, warp, lane, [&](int k, int ixy) {
+    shell_walk<SH_WARPS, SPLIT>(sh, T, rowpre, rowy0, n_cols, J.amp_scale, Wf, Wi, Wm, warp, lane, [&](int k, int ixy) {
         if (alpha != 1.0f) Wo[k] = __fmaf_rn(orient.y, T.D(Nx + (ixy >> 16)), orient.x * T.D(ixy & 0xFFFF));
     }, [&](int bl, float f, float rs, const float4& cf, int col, int, const float4& tz) {
         float amp = cf.z * tz.z * rs;
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
     row[32 * slots + lane] = carry;
 }
 
-template <int NM>
+template <int NM, bool SPLIT>
 int launch_cheb(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s, int* launched)
 {
     const size_t sm = (size_t)((t.max_axis_sum + 1) & ~1) * sizeof(float4) + (size_t)(NM + 1) * SH_RS * sizeof(int) +
@@ -300,13 +300,13 @@ int launch_cheb(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s, in
                       (size_t)SH_WARPS * 32 * (sizeof(float4) + sizeof(int2)) +
                       (size_t)SH_WARPS * (SHELL_MW * sizeof(unsigned) + 32 * sizeof(float));
     static std::atomic<unsigned long long> opened{0};
-    int rc = ism_open_smem((const void*)shell_kernel<NM>, &opened);
+    int rc = ism_open_smem((const void*)shell_kernel<NM, SPLIT>, &opened);
     if (rc) return rc;
     // all of the unified L1 as shared memory: 5 CTAs of ~27 KB per SM
-    cudaError_t e = cudaFuncSetAttribute(shell_kernel<NM>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    cudaError_t e = cudaFuncSetAttribute(shell_kernel<NM, SPLIT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return (int)e;
-    shell_kernel<NM><<<(unsigned)p.shell_ctas, SH_WARPS * 32, sm, s>>>(
+    shell_kernel<NM, SPLIT><<<(unsigned)p.shell_ctas, SH_WARPS * 32, sm, s>>>(
         t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<const float*>(ws + p.lut_off),
         reinterpret_cast<float*>(ws + p.rows_off));
     ++*launched;
@@ -319,14 +319,16 @@ int ism_launch_accum_cheb(const JobTable& t, const WsPlan& p, char* ws, void* st
 {
     *launched = 0;
     if (p.shell_ctas <= 0 || !t.any_cheb) return 0;
-    bool plain = false, wide = false;
+    bool plain[2] = {false, false}, wide[2] = {false, false};   // [split offsets]
     for (int i = 0; i < t.n_jobs; ++i) {
-        plain |= t.j[i].use_cheb == ISM_CHEB_NF;
-        wide |= t.j[i].use_cheb == ISM_CHEB_NW;
+        plain[shell_split(t.j[i])] |= t.j[i].use_cheb == ISM_CHEB_NF;
+        wide[shell_split(t.j[i])] |= t.j[i].use_cheb == ISM_CHEB_NW;
     }
     int rc = 0;
     cudaStream_t s = (cudaStream_t)stream;
-    if (plain) rc = launch_cheb<ISM_CHEB_NF>(t, p, ws, s, launched);
-    if (!rc && wide) rc = launch_cheb<ISM_CHEB_NW>(t, p, ws, s, launched);
+    if (plain[1]) rc = launch_cheb<ISM_CHEB_NF, true>(t, p, ws, s, launched);
+    if (!rc && plain[0]) rc = launch_cheb<ISM_CHEB_NF, false>(t, p, ws, s, launched);
+    if (!rc && wide[1]) rc = launch_cheb<ISM_CHEB_NW, true>(t, p, ws, s, launched);
+    if (!rc && wide[0]) rc = launch_cheb<ISM_CHEB_NW, false>(t, p, ws, s, launched);
     return rc;
 }

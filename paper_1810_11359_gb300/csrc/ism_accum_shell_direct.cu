@@ -50,14 +50,13 @@ namespace {
 __host__ __device__ __forceinline__ int sd_win(int B) { return 32 * B + 32; }
 __host__ __device__ __forceinline__ int sd_winp(int B) { return sd_win(B) + 32; }
 
-template <int PREC>
+template <int PREC, bool SPLIT>   // SPLIT: squared offsets in split form (ism_shell.cuh)
 __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __grid_constant__ JobTable t,
                                                                         const float4* __restrict__ tbl,
                                                                         const float* __restrict__ lut_g,
                                                                         float* __restrict__ rows, int winp)
 {
     constexpr bool HALF = PREC == PREC_FP16 || PREC == PREC_BF16;
-    constexpr bool SPLIT = PREC == PREC_FP32;   // squared offsets in split form (ism_shell.cuh)
     constexpr int LQ = ism_lut_phases(1);   // table phases per sample (LUT forms)
     constexpr int WIN = 64;   // window row of a bin: 32 (SLOTS + 1), SLOTS = 1
     extern __shared__ __align__(16) unsigned char smem[];
@@ -81,6 +80,7 @@ __global__ void __launch_bounds__(SD_WARPS * 32, 4) shell_direct_kernel(const __
         grp = t.j[jid].shell_groups - 1 - (int)(local % t.j[jid].shell_groups);
     }
     const JobDev& J = t.j[jid];
+    if (PREC == PREC_FP32 && shell_split(J) != SPLIT) return;   // the other instantiation's job (CTA-uniform)
     const int B = J.shell_direct;   // bins per shell: 8 (dense rooms) or 32 (sparse ones)
     const int q0 = grp * B;
     const int nb = min(B, J.Q - q0);
@@ -320,17 +320,17 @@ size_t shell_direct_smem(const JobTable& t)
 
 }  // namespace
 
-template <int PREC>
+template <int PREC, bool SPLIT>
 static int launch_sd(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s)
 {
     const size_t sm = shell_direct_smem(t);
     static std::atomic<unsigned long long> opened{0};
-    int rc = ism_open_smem((const void*)shell_direct_kernel<PREC>, &opened);
+    int rc = ism_open_smem((const void*)shell_direct_kernel<PREC, SPLIT>, &opened);
     if (rc) return rc;
-    cudaError_t e = cudaFuncSetAttribute(shell_direct_kernel<PREC>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    cudaError_t e = cudaFuncSetAttribute(shell_direct_kernel<PREC, SPLIT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return (int)e;
-    shell_direct_kernel<PREC><<<(unsigned)p.sd_ctas, SD_WARPS * 32, sm, s>>>(
+    shell_direct_kernel<PREC, SPLIT><<<(unsigned)p.sd_ctas, SD_WARPS * 32, sm, s>>>(
         t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<const float*>(ws + p.lut_off),
         reinterpret_cast<float*>(ws + p.rows_off), sd_winp(sd_bins_max(t)));
     return (int)cudaGetLastError();
@@ -342,16 +342,24 @@ int ism_launch_accum_shell_direct(const JobTable& t, const WsPlan& p, char* ws, 
     *launched = 0;
     if (p.sd_ctas <= 0) return 0;
     cudaStream_t s = (cudaStream_t)stream;
-    int rc;
+    int rc = 0, n = 1;
     switch (prec) {
     case ISM_PREC_FP32:
-    case ISM_PREC_FP32_DIRECT: rc = launch_sd<PREC_FP32>(t, p, ws, s); break;
-    case ISM_PREC_FP16X2: rc = launch_sd<PREC_FP16>(t, p, ws, s); break;
-    case ISM_PREC_BF16X2: rc = launch_sd<PREC_BF16>(t, p, ws, s); break;
-    case ISM_PREC_LUT: rc = launch_sd<PREC_LUT>(t, p, ws, s); break;
-    case ISM_PREC_LUT_TEX: rc = launch_sd<PREC_TEX>(t, p, ws, s); break;
+    case ISM_PREC_FP32_DIRECT: {
+        bool split[2] = {false, false};
+        for (int i = 0; i < t.n_jobs; ++i)
+            if (t.j[i].shell_direct) split[shell_split(t.j[i])] = true;
+        if (split[1]) rc = launch_sd<PREC_FP32, true>(t, p, ws, s);
+        if (!rc && split[0]) rc = launch_sd<PREC_FP32, false>(t, p, ws, s);
+        n = split[0] + split[1];
+        break;
+    }
+    case ISM_PREC_FP16X2: rc = launch_sd<PREC_FP16, false>(t, p, ws, s); break;
+    case ISM_PREC_BF16X2: rc = launch_sd<PREC_BF16, false>(t, p, ws, s); break;
+    case ISM_PREC_LUT: rc = launch_sd<PREC_LUT, false>(t, p, ws, s); break;
+    case ISM_PREC_LUT_TEX: rc = launch_sd<PREC_TEX, false>(t, p, ws, s); break;
     default: return (int)cudaErrorInvalidValue;
     }
-    *launched = rc ? 0 : 1;
+    *launched = rc ? 0 : n;
     return rc;
 }

@@ -49,7 +49,7 @@ namespace {
 #define SA_GV 3               // float4 per Gamma row (9 or 11 terms, padded)
 #define SA_NG 12              // gradient components: dp_r[3], dp_s[3], dbeta[6]
 
-template <int NT>
+template <int NT, bool SPLIT>
 __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const __grid_constant__ JobTable t,
                                                                           const float4* __restrict__ tbl,
                                                                           const float4* __restrict__ dtbl,
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     int jid, r, grp;
     if (!shell_cta(t, blockIdx.x, &jid, &r, &grp)) return;   // CTA-uniform
     const JobDev& J = t.j[jid];
-    if (J.adj_cheb != NT) return;   // another instantiation's job
+    if (J.adj_cheb != NT || shell_split(J) != SPLIT) return;   // another instantiation's job
     const int q0 = grp * SA_B;
     const int nb = min(SA_B, J.Q - q0);
     const int Nx = J.N[0], Ny = J.N[1];
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     const float4* Tg = tbl + J.tbl_base + (long long)r * n_axis;
     const float4* Xg = dtbl + J.tbl_base + (long long)r * n_axis;
     for (int e = threadIdx.x; e < n_axis; e += blockDim.x) {
-        shell_stage<true>(T, e, Tg[e], s2_magic);
+        shell_stage<SPLIT>(T, e, Tg[e], s2_magic);
         X[e] = Xg[e];
     }
     // dLoss/dh over the windows of the CTA's bins (bin q's: samples 32 q - H + P, P < 32 + 2 H; 0
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     for (int c = 0; c < SA_NG; ++c) G[c] = 0.0f;
     const float amp_scale = J.amp_scale;
     const float kfs = J.kfs_hi;   // f_s / c
-    shell_walk<SA_WARPS>(sh, T, rowpre, rowy0, n_cols, 1.0f, recf + warp * 32, Wi + warp * 32, Wm + warp * SHELL_MW, warp, lane,
+    shell_walk<SA_WARPS, SPLIT>(sh, T, rowpre, rowy0, n_cols, 1.0f, recf + warp * 32, Wi + warp * 32, Wm + warp * SHELL_MW, warp, lane,
                          [&](int k, int ixy) { Wx[k] = ixy; },
                          [&](int bl, float f, float rs, const float4& cf, int col, int ez, const float4& tz) {
         const float4* Gr = Gam + bl * SA_GV;   // [bin][offset], 32 offsets per bin
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32, 4) shell_adjoint_kernel(const _
     }
 }
 
-template <int NT>
+template <int NT, bool SPLIT>
 int launch_adj_cheb(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s, int max_taps)
 {
     const size_t axis_pad = (size_t)((t.max_axis_sum + 1) & ~1);
@@ -222,12 +222,12 @@ int launch_adj_cheb(const JobTable& t, const WsPlan& p, char* ws, cudaStream_t s
                       2 * rows * sizeof(int) + (size_t)SA_WARPS * 32 * (sizeof(float4) + sizeof(int2) + sizeof(int)) +
                       (size_t)SA_WARPS * SHELL_MW * sizeof(unsigned);
     static std::atomic<unsigned long long> opened{0};
-    int rc = ism_open_smem((const void*)shell_adjoint_kernel<NT>, &opened);
+    int rc = ism_open_smem((const void*)shell_adjoint_kernel<NT, SPLIT>, &opened);
     if (rc) return rc;
-    cudaError_t e = cudaFuncSetAttribute(shell_adjoint_kernel<NT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    cudaError_t e = cudaFuncSetAttribute(shell_adjoint_kernel<NT, SPLIT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          cudaSharedmemCarveoutMaxShared);   // 4 CTAs of ~32 KB per SM
     if (e != cudaSuccess) return (int)e;
-    shell_adjoint_kernel<NT><<<(unsigned)p.shell_ctas, SA_WARPS * 32, sm, s>>>(
+    shell_adjoint_kernel<NT, SPLIT><<<(unsigned)p.shell_ctas, SA_WARPS * 32, sm, s>>>(
         t, reinterpret_cast<const float4*>(ws + p.tbl_off), reinterpret_cast<const float4*>(ws + p.dtbl_off),
         reinterpret_cast<const float*>(ws + p.lut_off), reinterpret_cast<float*>(ws + p.gpart_off), max_taps);
     return (int)cudaGetLastError();
@@ -239,16 +239,20 @@ int ism_launch_adjoint_cheb(const JobTable& t, const WsPlan& p, char* ws, void* 
 {
     *launched = 0;
     if (p.shell_ctas <= 0) return 0;
-    bool plain = false, wide = false;
+    bool plain[2] = {false, false}, wide[2] = {false, false};   // [split offsets]
     int max_taps = 32;   // (a multiple of 4: the tables behind the window are 16-byte aligned)
     for (int i = 0; i < t.n_jobs; ++i) {
-        plain |= t.j[i].adj_cheb == ISM_CHEB_N;
+        const int split = shell_split(t.j[i]);
+        plain[split] |= t.j[i].adj_cheb == ISM_CHEB_N;
         if (t.j[i].adj_cheb != ISM_CHEB_AW) continue;
-        wide = true;
+        wide[split] = true;
         max_taps = std::max(max_taps, (2 * t.j[i].H + 3) & ~3);
     }
+    cudaStream_t s = (cudaStream_t)stream;
     int rc = 0;
-    if (plain) rc = launch_adj_cheb<ISM_CHEB_N>(t, p, ws, (cudaStream_t)stream, 32), ++*launched;
-    if (!rc && wide) rc = launch_adj_cheb<ISM_CHEB_AW>(t, p, ws, (cudaStream_t)stream, max_taps), ++*launched;
+    if (plain[1]) rc = launch_adj_cheb<ISM_CHEB_N, true>(t, p, ws, s, 32), ++*launched;
+    if (!rc && plain[0]) rc = launch_adj_cheb<ISM_CHEB_N, false>(t, p, ws, s, 32), ++*launched;
+    if (!rc && wide[1]) rc = launch_adj_cheb<ISM_CHEB_AW, true>(t, p, ws, s, max_taps), ++*launched;
+    if (!rc && wide[0]) rc = launch_adj_cheb<ISM_CHEB_AW, false>(t, p, ws, s, max_taps), ++*launched;
     return rc;
 }

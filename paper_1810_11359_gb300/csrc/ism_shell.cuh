@@ -103,10 +103,16 @@ struct Shell {
 // value and its rounding error.  G is a power of two with 2^24 G above every squared
 // delay of the RIR that a candidate can have (shell_s2_magic = 1.5 2^23 G), so the hi
 // parts of the three axes add without rounding and a sum of two entries is two FADDs
-// instead of a two-sum (ff_add: 10 operations).  |lo| <= G / 2, so the lo parts carry
-// an absolute error of a few 2^-24 G samples^2: below 2^-23 s relative to s^2 <= 2^24 G,
-// and at short delays a few 1e-7 sample at most.  Both subtractions are exact.  The
-// reduced tap arithmetics (SPLIT = false) keep the two-sum on the table as it is: a
+// instead of a two-sum (ff_add: 10 operations).  Both subtractions are exact; what is lost
+// are the low words of the lo parts, |lo| <= G / 2: a few 2^-25 G samples^2, or up to
+// 2^-24 G / s samples of a delay s, at most 2^-24 sqrt(G) near s = sqrt(G); relative to the
+// 2^-25 that f is rounded to it matters for the direct path of a long RIR.  Root mean squares
+// over directions, samples, 0.2 to 0.4 m from the source at 16 / 48 kHz (rounding alone:
+// 1.3e-8): G = 8 (11,300 samples) 1.5e-8 / 1.3e-8, 32 (22,600) 3.1e-8 / 1.6e-8, 256 (64,000)
+// 2.1e-7 / 7.6e-8, the largest 2.7e-7, 1.1e-7 and 1.3e-6.  So jobs of more than
+// ISM_SPLIT_SAMPLES samples (G > 32) keep the two-sum on the table as it is (SPLIT = false;
+// by job, since two shells must find the same integer delay for an image at their border).
+// The reduced tap arithmetics keep it at every length: a
 // change in the fraction's last bit can move a 16-bit tap by its own, far larger,
 // last bit.
 struct ShellTab {
@@ -127,6 +133,9 @@ __device__ __forceinline__ ShellTab shell_tab(unsigned char* smem, int max_axis_
     float* F = reinterpret_cast<float*>(s2 + n);
     return {s2, F, F + n};
 }
+
+// (of FP32 forms)
+__host__ __device__ inline bool shell_split(const JobDev& J) { return J.n_ism + J.H <= ISM_SPLIT_SAMPLES; }
 
 __device__ __forceinline__ float shell_s2_magic(const JobDev& J)
 {
@@ -264,8 +273,8 @@ static_assert(ISM_MAX_AXIS <= SHELL_MAX, "a column's candidates fit one pass");
 // correction from the exact residual hi - r^2 (FMA) + lo gives s = r + corr to ~2^-44
 // relative.  b is floor(r) moved by the floor of the corrected fraction; both floors
 // are additions of 1.5 2^23 rounded down, whose bits hold the integer (no conversion
-// unit).  b and f depend on the image alone, never on the shell, so every image lands
-// in exactly one shell.
+// unit).  b and f depend on the image and its job's length, never on the shell, so every
+// image lands in exactly one shell.
 template <bool SPLIT>
 __device__ __forceinline__ bool shell_delay(const Shell& sh, const ShellTab& T, const float4& cf, int2 ci, int j,
                                             int* bl_out, float* f_out, float* rs_out, int* ez_out, float4* tz_out)
@@ -352,7 +361,7 @@ __device__ __forceinline__ int shell_pass(const Shell& sh, const ShellTab& T, co
 // column's record (cf.z = col_scale F_x F_y), o = the record's place, where
 // extra(o, ix | iy << 16) was called before, ez, tz = its z entry in the tables.  Wf, Wi:
 // the warp's 32-entry scratch in shared memory; Wm: its SHELL_MW words.
-template <int WARPS, class X, class F>
+template <int WARPS, bool SPLIT, class X, class F>
 __device__ __forceinline__ void shell_walk(const Shell& sh, const ShellTab& T, const int* rowpre, const int* rowy0,
                                            int n_cols, float col_scale, float4* Wf, int2* Wi, unsigned* Wm, int warp, int lane,
                                            X&& extra, F&& on_image)
@@ -362,7 +371,7 @@ __device__ __forceinline__ void shell_walk(const Shell& sh, const ShellTab& T, c
         int total, base = 0;
         do {   // (one pass but for very flat rooms)
             int start, cnt, k;
-            const int n = shell_pass<true>(sh, T, rowpre, rowy0, n_cols, c0, base, col_scale, Wf, Wi, Wm, lane, &total,
+            const int n = shell_pass<SPLIT>(sh, T, rowpre, rowy0, n_cols, c0, base, col_scale, Wf, Wi, Wm, lane, &total,
                                            &start, &cnt, &k, extra);
             __syncwarp();
             int cols = -1;   // last column begun before the batch
@@ -376,7 +385,7 @@ __device__ __forceinline__ void shell_walk(const Shell& sh, const ShellTab& T, c
                     int bl, ez;
                     float f, rs;
                     float4 tz;
-                    if (shell_delay<true>(sh, T, cf, Wi[o], j, &bl, &f, &rs, &ez, &tz))
+                    if (shell_delay<SPLIT>(sh, T, cf, Wi[o], j, &bl, &f, &rs, &ez, &tz))
                         on_image(bl, f, rs, cf, o, ez, tz);
                 }
             }
