@@ -68,10 +68,13 @@
 // fills (cheb_table), and the expansion takes 32 taps at a time, each turn's
 // upper half carried into the next.  The terms are converted to integers
 // (cvt.rni) instead of rounded by the FFMA, which lifts the 2^22 cap on a
-// term: with few images per integer delay the sums then hold up to 30 bits of
-// a term, and a sparse RIR's error stays at the per-tap sum's (3.6e-7 of its
-// norm with the cap, 1.6e-7 without it, 1.4e-7 per tap, 15 RIRs of 176 taps),
-// at no cost in time (the conversions go to a unit that is 14 % busy).
+// term: with few images per integer delay the sums then hold up to 30 bits of a
+// term, at no cost in time (the conversions go to a unit that is 14 % busy), and the
+// expansion adds its terms from the last, smallest one on, c_0 (the same for every
+// image) in two parts.  A RIR's error is then no larger than the per-tap sum's (of its
+// norm, 15 RIRs of 176 taps, sparse: 3.6e-7 with the cap on a term, 1.7e-7 without it,
+// 1.4e-7 now, 1.5e-7 per tap; of 64 taps in two dense rooms 1.27 and 1.19e-7 before,
+// 0.95 and 0.91e-7 now, 1.18 and 1.08e-7 per tap).
 #include "ism_accum.cuh"
 #include "ism_shell.cuh"
 
@@ -268,6 +271,7 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
 #pragma unroll
         for (int i = 0; i < NM; ++i)
             c[i] = NM == ISM_CHEB_NF ? t.cheb[lane * ISM_CHEB_N + i] : tabs[J.lut_base + (i * slots + sl) * 32 + lane];
+        const float c0_lo = CVT ? tabs[J.lut_base + (NM * slots + sl) * 32 + lane] : 0.0f;
         float acc[2] = {carry, 0.0f};
         for (int o = 0; o < SH_NO; ++o) {
             if (!((nonempty >> o) & 1u)) continue;   // warp-uniform
@@ -281,9 +285,15 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) shell_kernel(const __grid_co
                 mv[4 * v + 3] = w.w;
             }
             float D[1];
-            D[0] = c[0] * mv[0];
+            if constexpr (CVT) {   // the small terms first
+                D[0] = c0_lo * mv[0];
 #pragma unroll
-            for (int k = 1; k < NM; ++k) D[0] = __fmaf_rn(c[k], mv[k], D[0]);
+                for (int k = NM - 1; k >= 0; --k) D[0] = __fmaf_rn(c[k], mv[k], D[0]);
+            } else {               // (held to the truncation of 4e-7 in any order)
+                D[0] = c[0] * mv[0];
+#pragma unroll
+                for (int k = 1; k < NM; ++k) D[0] = __fmaf_rn(c[k], mv[k], D[0]);
+            }
             flush_run<1, false>(D, acc, o - 1, lane, 1.0f);
         }
         row[32 * sl + lane] = acc[0];

@@ -77,7 +77,9 @@ __device__ void cheb_table(const JobDev& J, int N, int tap0, float* tab)
             q = q > 2 * N ? 4 * N - q : q;
             c += gv[e % 8][k] * (q > N ? -cs[2 * N - q] : cs[q]);
         }
-        tab[i * 32 * J.slots + t] = (float)(c * (i == 0 ? inv_s : 2.0 * inv_s));
+        c *= i == 0 ? inv_s : 2.0 * inv_s;
+        tab[i * 32 * J.slots + t] = (float)c;
+        if (i == 0) tab[N * 32 * J.slots + t] = (float)(c - (double)(float)c);   // the rest of c_0, after the terms
     }
 }
 

@@ -58,7 +58,7 @@
 #define ISM_CHEB_AW 11            // terms of the adjoint for windows other than 32 taps (degree 10)
 #define ISM_CHEB_MAX 12           // terms of any of them, at most
 #define ISM_ADJ_MIN_NW 80         // windows that end inside a sample interval: shortest for the fused adjoint
-#define ISM_CHEB_TAB 4096         // floats of a coefficient table in the workspace: [term][32 slots]
+#define ISM_CHEB_TAB 4096         // floats of a coefficient table in the workspace: [term, rest of c_0][32 slots]
 #define ISM_CHEB_TAB_CTAS 32      // CTAs that fill one (8 taps each)
 #define ISM_SHELL_BINS 8          // delay bins per CTA of the fused Chebyshev accumulation
 #define ISM_SD_BINS 32            // delay bins per CTA of the fused direct accumulation

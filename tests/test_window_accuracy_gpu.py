@@ -34,8 +34,8 @@ def _errors(taps, prec, n_rir=6):
     Tw = float(np.float32(taps / FS))
     N = oracle.nb_img_from_t(T, ROOM, 343.0, Tw)
     got = ism.ism_simulate(ROOM, BETA, ps, pr, N, T, FS, Tw=Tw, prec=prec).cpu().numpy().astype(np.float64)[:, 0]
-    ref = np.stack([oracle.rir(ROOM, BETA.astype(np.float64), 343.0, FS, Tw, p.astype(np.float64), pr[0].astype(np.float64), N,
-                               got.shape[-1]) for p in ps])
+    ref = oracle.rir_list(ROOM, BETA.astype(np.float64), 343.0, FS, Tw, ps.astype(np.float64),
+                          np.broadcast_to(pr[0].astype(np.float64), ps.shape), N, got.shape[-1])
     return np.linalg.norm(got - ref, axis=1) / np.linalg.norm(ref, axis=1)
 
 
@@ -44,3 +44,10 @@ def _errors(taps, prec, n_rir=6):
 @pytest.mark.parametrize("taps", [16.0, 16.8, 17.5, 18.0, 18.8, 20.8, 24.8, 28.8, 33.3, 40.5, 44.1, 50.7, 63.2, 64.0, 79.0, 81.0])
 def test_dense_windows(taps):
     assert np.sqrt(np.mean(_errors(taps, "fp32") ** 2)) <= 2e-7
+
+
+def test_series_has_no_more_error_than_the_taps_one_by_one():
+    """Windows that go through the series, over lengths whose rounded coefficients differ."""
+    taps = [16.0, 18.0, 24.0, 36.0, 44.0, 50.0, 64.0, 82.5, 88.2, 96.7, 110.25, 128.0, 150.3, 176.4, 192.0, 224.5]
+    series, direct = (np.concatenate([_errors(t, p) for t in taps]) for p in ("fp32", "fp32_direct"))
+    assert np.mean(series ** 2) <= np.mean(direct ** 2)
