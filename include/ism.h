@@ -118,6 +118,9 @@ const char* ism_status_string(ism_status s);
 const char* ism_last_error_message(void);
 /* ISM_VERSION of the loaded library. */
 int ism_version(void);
+/* Launch graphs captured and replayed by this process so far (ism_simulate_host,
+ * ism_simulate_batch); either pointer may be NULL.  Host only. */
+void ism_launch_graph_counts(long long* captured, long long* replayed);
 
 /* ------------------------------------------------------------------------- */
 /* Sizing                                                                     */
@@ -175,11 +178,13 @@ ism_status ism_simulate(const ism_room* room, const float* pos_src, int n_src, c
  * than the positions' values -- room, counts, nb_img, times, fs, prec, seed, a
  * page-locked `out`, workspace and its size, the device and the ism_set_lanes()
  * setting -- equal an earlier call's replays a CUDA graph of that call's
- * launches, captured once after it ran (into other memory: after the second such
+ * launches, captured once after it ran (into other memory: after the fourth such
  * call; the positions are copied into the workspace first and the result out of
  * it, as always): bit-identical results, without the planning and the
- * per-launch parameter copies.  The library keeps the 16 most
- * recently used graphs (each holds its launches' 32 KB job tables); they hold the
+ * per-launch parameter copies.  The library keeps 16
+ * graphs (each holds its launches' 32 KB job tables); a new one takes the place of
+ * the least recently used if the last 64 calls did not use that, and otherwise its
+ * calls run as the first did.  The graphs hold the
  * workspace and `out` addresses, so freeing either and calling again with the
  * same addresses is fine, and per-device state ends with cudaDeviceReset. */
 ism_status ism_simulate_host(const ism_room* room, const float* pos_src, int n_src,

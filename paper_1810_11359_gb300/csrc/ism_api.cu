@@ -1139,29 +1139,40 @@ ism_status ism_fail_message(ism_status s, const char* fmt, ...)
 // replays the CUDA graph of that call's launches instead of building the job tables
 // and the plan and issuing the dozen launches with their 32 KB parameter tables
 // again.  The graph is captured (nothing runs while capturing) after a call ran
-// eagerly: the host entry captures after its first call (when the kernels write its
-// page-locked result themselves) or when a key comes back (when the result is copied:
-// 4 RIRs with a tail 87 -> 63 us a call), ism_simulate_batch when a key comes back (so that
+// eagerly: the host entry captures after its first call when the kernels write its
+// page-locked result themselves, and after the fourth when the result is copied: 4 RIRs
+// with a tail take 108 us eagerly, 66 replayed, and a capture with the first launches of
+// its graph 120 more, three calls' gain.  ism_simulate_batch captures when a key comes back (so that
 // a stream of distinct batches, as the server's, pays nothing but the key).  Calls
 // on a stream being captured by the caller, calls
 // while the stage profiler runs, and jobs with device-resident coefficients run
-// eagerly.  At most HG_MAX graphs are kept (the least recently used one goes); the
-// lookup and the launch hold one lock, so no thread destroys a graph another is
+// eagerly.  At most HG_MAX graphs are kept.  A new one takes the place of the least
+// recently used, and only of one that the last HG_IDLE lookups did not use: more keys in
+// turn than graphs keep the graphs there are, the others running eagerly, where each
+// would push out the next one to be used (20 rooms in turn 90 -> 81 us a call, 32 rooms
+// 140 -> 109; 108 without graphs).
+// The lookup and the launch hold one lock, so no thread destroys a graph another is
 // about to launch.
 namespace {
 #define HG_MAX 16
 #define HG_SEEN 32
+#define HG_IDLE 64   // (above HG_MAX + HG_SEEN: the keys in turn that can come back at all)
 struct HostGraph {
     std::string key;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t x = nullptr;
     size_t pos_off = 0;   // host entry: where the positions go in the workspace
-    unsigned long long tick = 0;
+    unsigned long long tick = 0;   // lookup that used it last
+};
+struct SeenKey {
+    std::string key;
+    int calls;
 };
 std::mutex g_hg_mu;
 std::vector<HostGraph> g_hg;
-std::vector<std::string> g_hg_seen;   // keys met once (ism_simulate_batch), most recent last
-unsigned long long g_hg_tick = 0;
+std::vector<SeenKey> g_hg_seen;   // keys met but not captured, most recent last
+unsigned long long g_hg_tick = 0;   // lookups
+long long g_hg_captured = 0, g_hg_replayed = 0;
 
 template <class T>
 void key_put(std::string& k, const T& v)
@@ -1251,29 +1262,45 @@ int hg_replay(const std::string& key, cudaStream_t st, Pre pre, bool* hit)
 {
     *hit = false;
     std::lock_guard<std::mutex> g(g_hg_mu);
+    ++g_hg_tick;
     for (HostGraph& h : g_hg) {
         if (h.key != key) continue;
-        h.tick = ++g_hg_tick;
+        h.tick = g_hg_tick;
         int e = pre(h.pos_off);
         if (!e) e = (int)cudaGraphLaunch(h.x, st);
         *hit = e == 0;
+        g_hg_replayed += e == 0;
         return e;
     }
     return 0;
 }
 
-// Whether a batch key came before (and remember it): the batch entry captures on the
-// second sighting.
-bool hg_seen_before(const std::string& key)
+// The graph that a new one takes the place of (g_hg.size(): none has to go; -1: all are
+// in use).  Under the lock.
+int hg_place()
+{
+    if (g_hg.size() < HG_MAX) return (int)g_hg.size();
+    size_t old = 0;
+    for (size_t i = 1; i < g_hg.size(); ++i)
+        if (g_hg[i].tick < g_hg[old].tick) old = i;
+    return g_hg_tick - g_hg[old].tick > HG_IDLE ? (int)old : -1;
+}
+
+// Whether a key without a graph has now come `calls` times (and remember it), and there is a
+// place for its graph.
+bool hg_due(const std::string& key, int calls)
 {
     std::lock_guard<std::mutex> g(g_hg_mu);
+    SeenKey k{key, 0};
     for (size_t i = 0; i < g_hg_seen.size(); ++i)
-        if (g_hg_seen[i] == key) {
+        if (g_hg_seen[i].key == key) {
+            k = g_hg_seen[i];
             g_hg_seen.erase(g_hg_seen.begin() + (long)i);
-            return true;
+            break;
         }
+    if (++k.calls >= calls && hg_place() >= 0) return true;
     if (g_hg_seen.size() >= HG_SEEN) g_hg_seen.erase(g_hg_seen.begin());
-    g_hg_seen.push_back(key);
+    g_hg_seen.push_back(k);
     return false;
 }
 
@@ -1286,25 +1313,25 @@ void hg_store(const std::string& key, size_t pos_off, Run run)
     cudaGraph_t g = nullptr;
     cudaGraphExec_t x = nullptr;
     std::lock_guard<std::mutex> lk(g_hg_mu);
+    const int place = hg_place();
+    if (place < 0) return;
     if (capture_stream(&cs) == 0 && cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         const ism_status sc = run(cs);
         const cudaError_t ec = cudaStreamEndCapture(cs, &g);
         if (sc == ISM_OK && ec == cudaSuccess && g && cudaGraphInstantiate(&x, g, 0) == cudaSuccess) {
-            if (g_hg.size() >= HG_MAX) {
-                size_t old = 0;
-                for (size_t i = 1; i < g_hg.size(); ++i)
-                    if (g_hg[i].tick < g_hg[old].tick) old = i;
-                cudaGraphExecDestroy(g_hg[old].x);
-                cudaGraphDestroy(g_hg[old].g);
-                g_hg.erase(g_hg.begin() + (long)old);
+            if (place < (int)g_hg.size()) {
+                cudaGraphExecDestroy(g_hg[place].x);
+                cudaGraphDestroy(g_hg[place].g);
+                g_hg.erase(g_hg.begin() + place);
             }
             HostGraph h;
             h.key = key;
             h.g = g;
             h.x = x;
             h.pos_off = pos_off;
-            h.tick = ++g_hg_tick;
+            h.tick = g_hg_tick;
             g_hg.push_back(h);
+            ++g_hg_captured;
         } else if (g) {
             cudaGraphDestroy(g);
         }
@@ -1336,6 +1363,13 @@ const char* ism_status_string(ism_status s)
 const char* ism_last_error_message(void) { return g_last_error.c_str(); }
 
 int ism_version(void) { return ISM_VERSION; }
+
+void ism_launch_graph_counts(long long* captured, long long* replayed)
+{
+    std::lock_guard<std::mutex> g(g_hg_mu);
+    if (captured) *captured = g_hg_captured;
+    if (replayed) *replayed = g_hg_replayed;
+}
 
 ism_status ism_rir_length(float T, float fs, int* n_samples)
 {
@@ -1398,7 +1432,7 @@ ism_status ism_simulate_batch(const ism_job* jobs, int n_jobs, ism_precision pre
     std::vector<Validated> vs;
     if ((s = validate_all(jobs, n_jobs, vs, true)) != ISM_OK) return s;
     if ((s = run_batch(vs, prec, workspace, ws_bytes, stream)) != ISM_OK) return s;
-    if (!gkey.empty() && hg_seen_before(gkey))
+    if (!gkey.empty() && hg_due(gkey, 2))
         hg_store(gkey, 0, [&](cudaStream_t cs) { return run_batch(vs, prec, workspace, ws_bytes, cs); });
     return ISM_OK;
 }
@@ -1550,9 +1584,9 @@ ism_status ism_simulate_host(const ism_room* room, const float* pos_src, int n_s
     const HostCopy hc{d_out, out};
     if ((s = run_batch(vs, prec, workspace, sim, stream, direct ? nullptr : &hc)) != ISM_OK) return s;
     if ((e = (int)cudaStreamSynchronize(st))) return cuda_fail(e, "stream synchronize");
-    // capture this call's launches for the next identical one (a copied result: when a call
-    // comes back, and if it runs as one set of launches)
-    if (!gkey.empty() && (direct || (schedule(vs, prec, true).lanes == 1 && hg_seen_before(gkey))))
+    // capture this call's launches for the next identical one (a copied result: when it has
+    // come four times, and if it runs as one set of launches)
+    if (!gkey.empty() && (direct || (hg_due(gkey, 4) && schedule(vs, prec, true).lanes == 1)))
         hg_store(gkey, pos_off, [&](cudaStream_t cs) { return run_batch(vs, prec, workspace, sim, cs, nullptr); });
     return ISM_OK;
 }

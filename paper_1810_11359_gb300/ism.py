@@ -85,6 +85,7 @@ _SIGS = {
     "ism_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "ism_last_error_message": (ctypes.c_char_p, []),
     "ism_version": (ctypes.c_int, []),
+    "ism_launch_graph_counts": (None, [ctypes.POINTER(ctypes.c_longlong)] * 2),
     "ism_rir_length": (ctypes.c_int, [ctypes.c_float, ctypes.c_float, _P(ctypes.c_int)]),
     "ism_workspace_size": (ctypes.c_int, [_P(ism_room), ctypes.c_int, ctypes.c_int, _P(ctypes.c_int), ctypes.c_float,
                                           ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_int,
@@ -582,6 +583,13 @@ def ism_simulate_backward(L, beta, pos_src, pos_rcv, nb_img, Tmax, fs, grad_out,
     gj = make_grad_job(job, go, gb, gs, gr)
     ism_simulate_backward_batch([gj], workspace=workspace, stream=stream)
     return gb, gs, gr
+
+
+def ism_launch_graph_counts():
+    """(captured, replayed): launch graphs of repeated calls so far in this process."""
+    c, r = ctypes.c_longlong(), ctypes.c_longlong()
+    load().ism_launch_graph_counts(ctypes.byref(c), ctypes.byref(r))
+    return c.value, r.value
 
 
 AURALIZE_METHODS = {"auto": 0, "direct": 1, "fft": 2}
