@@ -554,7 +554,12 @@ ism_status validate_all(const ism_job* jobs, int n_jobs, std::vector<Validated>&
 // launch set.  Others run as one: the fused kernels leave the second half
 // nothing to overlap with, and halves have two last waves (a call, two halves
 // against one: 128 RIRs FP32 382 and 379 us, 64 RIRs FP16X2 629 and 566 us, 16
-// RIRs of 64 taps 352 and 320 us, 512 RIRs at 48 kHz 302 both).  A sub-job
+// RIRs of 64 taps 352 and 320 us, 512 RIRs at 48 kHz 302 both).  Where the lanes
+// alternate -- more than a set's worth of jobs -- the sets hold half as many jobs, so
+// that the two in flight take one full set's workspace and not two (128 rooms x 16
+// microphones, 32 taps, 0.6 s: 84 MB, 167 with full sets, 5240 us both; images to 0.25 s
+// 35 and 70 MB, 1096 and 1090 us; 300 x 8 of these 17 and 35 MB, 1372 and 1345); jobs of
+// a single RIR keep full sets (128 x 1: 407 us, 458 in halves).  A sub-job
 // keeps the RIR index of its first RIR (the noise counter), so every RIR is
 // computed exactly as in the unsplit job.
 struct Schedule {
@@ -580,8 +585,11 @@ bool sets_fit(const std::vector<Validated>& vs, ism_precision prec)
 Schedule schedule(const std::vector<Validated>& vs, ism_precision prec, bool copies)
 {
     Schedule sc;
-    double work = 0.0;
-    for (const Validated& v : vs) work += images_in_reach(v) * (double)v.job.n_src * v.job.n_rcv;
+    double work = 0.0, rirs = 0.0;
+    for (const Validated& v : vs) {
+        rirs += (double)v.job.n_src * v.job.n_rcv;
+        work += images_in_reach(v) * (double)v.job.n_src * v.job.n_rcv;
+    }
     const bool split = work >= 2.0e7 && g_lanes.load() >= 2 && (copies || !sets_fit(vs, prec));
     std::vector<Validated> halves[2];
     for (const Validated& v : vs) {
@@ -613,9 +621,14 @@ Schedule schedule(const std::vector<Validated>& vs, ism_precision prec, bool cop
             halves[part].push_back(w);
         }
     }
+    size_t per_set = ISM_MAX_JOBS;
+    if (!split && work >= 2.0e7 && g_lanes.load() >= 2 && vs.size() > ISM_MAX_JOBS && rirs >= 2.0 * vs.size()) {
+        const size_t n_sets = 2 * ((vs.size() + ISM_MAX_JOBS - 1) / ISM_MAX_JOBS);
+        per_set = (vs.size() + n_sets - 1) / n_sets;
+    }
     for (int part = 0; part < 2; ++part)
-        for (size_t g = 0; g < halves[part].size(); g += ISM_MAX_JOBS) {
-            const size_t e = std::min(halves[part].size(), g + ISM_MAX_JOBS);
+        for (size_t g = 0; g < halves[part].size(); g += per_set) {
+            const size_t e = std::min(halves[part].size(), g + per_set);
             sc.sets.emplace_back(halves[part].begin() + g, halves[part].begin() + e);
         }
     sc.lanes = (sc.sets.size() >= 2 && g_lanes.load() >= 2) ? 2 : 1;
