@@ -272,7 +272,7 @@ __device__ __forceinline__ unsigned long long pk_all(float a) { return pk_pack(a
 // Markstein's sequence (IBM J. Res. Dev. 34, 1990) -- a reciprocal refined once, the
 // quotient and its exact remainder by FMAs -- with every sign turned, so that no
 // negation is an instruction.  Checked against / for every argument that the
-// noise gives it (all 2^23 uniforms; tests).
+// noise gives it (all 2^23 uniforms, in either half: test_noise_all_uniforms_gpu.py).
 __device__ __forceinline__ unsigned long long pk_neg_div(unsigned long long a, unsigned long long b)
 {
     float b0, b1;
