@@ -10,8 +10,10 @@
 // 8, the least that holds the call's).  Lane l of a warp owns the outputs
 // T0 + 4 l + r, r = 0 .. 3, for the microphones (32 accumulators for 8).  For one
 // segment the taps k that connect it to the tile are walked in chunks of 128;
-// the chunks of all segments are dealt to the CTA's 16 warps in turn, which add
-// their partial sums in warp order at the end.  (16 points x 1 microphone, RIRs
+// the chunks of all segments are dealt to the CTA's warps in turn, which add
+// their partial sums in warp order at the end.  A segment's chunks are of one size (142 taps
+// as 72 + 70, not 128 + 14, of which every other warp would take the short ones: 18 segments
+// of 14 samples, RIRs of 27,800, 9 microphones 103 -> 74 us).  (16 points x 1 microphone, RIRs
 // of 9600 samples, a signal of 57,600: 337 us with 8 microphones' sums always
 // and whole segments dealt to 4 warps, 49 us now; 30 x 5, 16,000, 48,000: 340 ->
 // 282; the 48 kHz array 1285 -> 1193.)
@@ -67,7 +69,7 @@ __device__ __forceinline__ int au_start(int p, int n_x, int n_points, const int*
 
 // VEC: 128-bit tap staging (16-byte aligned RIR rows); AU_M: microphones per CTA
 template <bool VEC, int AU_M, int AU_WARPS>
-__global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS == 4 ? 6 : 1)
+__global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS > 4 ? 1 : AU_M == 8 ? 5 : 6)   // (8 in 80 registers: spills)
     auralize_kernel(const float* __restrict__ x, int n_x, const float* __restrict__ h, int n_points, int n_mics, int n_s,
                     const int* __restrict__ starts, float* __restrict__ y, int n_out)
 {
@@ -106,12 +108,15 @@ __global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS == 4 ? 6 : 1)
             const long long k_hi = min(T0 + AU_TILE - 1 - a, (long long)n_s - 1);
             if (k_hi < k_lo) continue;
             const float* hp = h + (long long)p * n_mics * n_s;
-            const int n_ch = (int)((k_hi - k_lo) / AU_KC) + 1;
+            const int n_k = (int)(k_hi - k_lo);
+            const int n_ch = n_k / AU_KC + 1;
+            const int kc = (n_k / n_ch + 4) & ~3;   // taps of a chunk: as even as whole groups allow
             const int first = (warp - turn + AU_WARPS) % AU_WARPS;   // the warp's first chunk of this segment
             turn = (turn + n_ch) % AU_WARPS;
-            for (long long k0 = k_lo + (long long)first * AU_KC; k0 <= k_hi; k0 += AU_WARPS * AU_KC) {
+            for (long long k0 = k_lo + (long long)first * kc; k0 <= k_hi; k0 += AU_WARPS * kc) {
                 __syncwarp();
-                // taps k0 .. k0 + KC - 1 of the microphones (0 past k_hi or past the array)
+                // taps k0 .. k0 + KC - 1 of the microphones (0 past k_hi or past the array; those
+                // past k0 + kc - 1 are not used)
                 if (VEC) {
                     for (int e = lane; e < AU_M * AU_KC / 4; e += 32) {   // 32 lanes: 512 contiguous bytes
                         const int m = e / (AU_KC / 4), kq = e % (AU_KC / 4);
@@ -143,8 +148,8 @@ __global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS == 4 ? 6 : 1)
                 // 4 l + KC - 4 - 4 g, xb4 = the next float4 (the previous group's xa)
                 const float4* xl = W.x + lane + (AU_KC - 4) / 4;
                 float4 xb4 = xl[1];
-                // the groups that hold taps <= k_hi (the last chunk of a segment is partial)
-                const int ng = (int)min((long long)(AU_KC / 4), (k_hi - k0) / 4 + 1);
+                // the groups that hold taps of the chunk
+                const int ng = (int)min((long long)(kc / 4), (k_hi - k0) / 4 + 1);
 #pragma unroll 2
                 for (int g = 0; g < ng; ++g) {
                     const float4 xa = xl[-g];
@@ -182,7 +187,7 @@ __global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS == 4 ? 6 : 1)
     __syncthreads();
     // thread e writes output (t, m) pairs; consecutive threads take consecutive t
     for (int e = threadIdx.x; e < AU_TILE * AU_M; e += blockDim.x) {
-        const int m = e / AU_TILE, i = e % AU_TILE;   // i = 8 l + r
+        const int m = e / AU_TILE, i = e % AU_TILE;   // i = 4 l + r
         const int l = i / AU_R, r = i % AU_R;
         float v = red[((0 * AU_R + r) * AU_M + m) * 32 + l];
 #pragma unroll
