@@ -1669,12 +1669,13 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
 // direct: about 4 N log2 N lane operations per length-N DFT (one per segment, one per
 // microphone pair and point, one inverse per pair) and 4 per product of spectra (8.0 T/s)
 // against n_mics n_x n_S multiply-adds (20.5 T/s).  Overlap-save, where its plan exists,
-// as the plan says, against the multiply-adds that the direct kernel issues: microphones
-// padded to 1, 2, 4 or 8 a CTA, a segment's taps to whole chunks of 128 for every tile of
-// 128 outputs (14 to 22 T/s of them; 1 microphone 9 to 14).  Direct and overlap-save, us:
+// as the plan says, against the multiply-adds of the direct form with microphones
+// padded to 1, 2, 4 or 8 a CTA and a segment's taps to whole chunks of 128 for every tile of
+// 128 outputs (17 T/s of them, 1 microphone 11; 5 us).  Over 410 sizes the choice takes 0.4 %
+// more than the better of the two on average, 37 % at most.  Direct and overlap-save, us:
 // 64 points x 2 microphones, RIRs of 4800 samples, 54 and 42; 941 x 8, 4858, segments of
-// 128 samples, 489 and 205; 100 x 1, 4800, 45 and 43.  892 x 2, whose piece spectra do not
-// fit: 206 direct, 4370 four-step.
+// 128 samples, 489 and 205; 100 x 1, 4800, 45 and 43; 1 x 1, 1000, a signal of 3438, 6 and 27.
+// 892 x 2, whose piece spectra do not fit: 206 direct, 4370 four-step.
 static int auralize_form(int n_x, int n_points, int n_mics, int n_S, bool uniform, int method, AfPlan* af,
                          size_t* af_need, AoPlan* ao)
 {
@@ -1693,13 +1694,13 @@ static int auralize_form(int n_x, int n_points, int n_mics, int n_S, bool unifor
     const double fft =
         ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * af->logN + (double)n_points * pairs * 4.0 * N;
     const double direct = (double)n_mics * (double)n_x * (double)n_S;
-    if (direct > 2.55 * fft) return fft_form;
+    if (!ols) return direct > 2.55 * fft ? ISM_AURALIZE_FORM_FOUR_STEP : ISM_AURALIZE_FORM_DIRECT;
     const double len = (double)n_x / n_points;
     const double padded = std::ceil((len + 127.0) / 128.0) * 128.0 / len;
     const int mics = n_mics <= 2 ? n_mics : n_mics <= 4 ? 4 : (n_mics + 7) / 8 * 8;
     const double issued = (double)mics * (double)n_x * (double)n_S * padded;
-    return ols && 1.0e-5 + issued / (mics == 1 ? 1.4e13 : 2.05e13) > ao->seconds ? ISM_AURALIZE_FORM_OVERLAP_SAVE
-                                                                                 : ISM_AURALIZE_FORM_DIRECT;
+    return 5.0e-6 + issued / (mics == 1 ? 1.1e13 : 1.7e13) > ao->seconds ? ISM_AURALIZE_FORM_OVERLAP_SAVE
+                                                                        : ISM_AURALIZE_FORM_DIRECT;
 }
 
 static ism_status auralize_args(const float* signal, int n_x, const float* rirs, int n_points, int n_mics, int n_S,

@@ -60,6 +60,15 @@ def test_automatic_choice_never_takes_the_four_step_form_for_overlap_saves_time(
             assert M * n_x * n_s > 2.55 * ops, (n_x, P, M, n_s, given)
 
 
+@pytest.mark.parametrize("size,given,form", [
+    ((270, 99, 2, 16285), True, "direct"),         # its 99 pieces would follow one another on 5 CTAs
+    ((541, 510, 9, 26015), True, "overlap_save"),  # 510 on 35, and the direct form slower still
+    ((3438, 1, 1, 1000), True, "direct"),          # less than three launches
+    ((4963, 88, 8, 9000), False, "overlap_save")])
+def test_automatic_choice_counts_the_pieces_that_follow_one_another(size, given, form):
+    assert ism.ism_auralize_form(*size, given_starts=given) == form
+
+
 @pytest.mark.parametrize("size", [(57600, 64, 8, 57600), (57600, 64, 2, 4800), (30000, 64, 4, 3200), (144000, 500, 2, 19200)])
 def test_workspace_of_the_overlap_save_form(size):
     """The automatic choice asks for the overlap-save form's piece spectra (18 KB each; of given
