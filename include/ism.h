@@ -87,7 +87,7 @@ typedef enum {
  *   the 32 taps.  Other windows use the direct evaluation of
  *   ISM_PREC_FP32_DIRECT. */
 typedef enum {
-    ISM_PREC_FP32 = 0,        /* FP32, Chebyshev moments (32-tap windows), else direct */
+    ISM_PREC_FP32 = 0,        /* FP32, Chebyshev moments in dense rooms, else direct */
     ISM_PREC_FP16X2 = 1,      /* packed FP16 window and sinc, FP32 accumulation        */
     ISM_PREC_BF16X2 = 2,      /* packed BF16 window and sinc, FP32 accumulation; BF16's
                                * 8-bit significand bounds its error only to ~1e-2 of

@@ -5,8 +5,9 @@
 int ism_launch_accum(const JobTable& t, const WsPlan& p, char* ws, ism_precision prec, void* stream,
                      void* direct_stream, int* launched)
 {
-    // the fused kernels (32-tap windows: Chebyshev moments or every tap evaluated), then
-    // the per-tap kernel over binned ids for the other windows
+    // the fused kernels (every tap evaluated: 32-tap windows; Chebyshev moments: dense FP32
+    // bins of the windows that a series follows), then the per-tap kernel over binned ids for
+    // the rest (see plan())
     int a = 0, b = 0, c = 0;
     int rc = ism_launch_accum_shell_direct(t, p, ws, prec, direct_stream, &b);
     if (!rc) rc = ism_launch_accum_cheb(t, p, ws, stream, &a);

@@ -1031,9 +1031,10 @@ ism_status run_batch(const std::vector<Validated>& vs, ism_precision prec, void*
     return first_err;
 }
 
-// Backward pass: the forward's geometry; for 32-tap windows the fused
-// Chebyshev adjoint (which enumerates its own images), for other windows the
-// forward's enumeration and binning and the per-tap adjoint; then the
+// Backward pass: the forward's geometry; the fused Chebyshev adjoint (which
+// enumerates its own images) for windows of 32 taps, of any whole even number from
+// ISM_CHEB_MIN_NW on and of any length from ISM_ADJ_MIN_NW on, the forward's
+// enumeration and binning and the per-tap adjoint for the rest; then the
 // fixed-order reductions.
 ism_status run_backward(const std::vector<Validated>& vs, void* workspace, size_t ws_bytes, void* stream)
 {

@@ -13,7 +13,8 @@
 //             geometry launch unless the window has 32 taps) or tap by tap (32-tap
 //             windows: FP32 with sparse bins, the other tap arithmetics).  A set that
 //             holds both runs them on two streams.
-//   Jobs of neither (other windows: sparse bins, under 16 taps, reduced arithmetics):
+//   Jobs of neither (other windows: sparse bins, lengths that no series follows, the other
+//   tap arithmetics):
 //   enum(a)   per RIR and range of grid columns: delays of the images in reach, culling
 //             of those whose window misses [0, n_ism), counts per 32-sample delay bin.
 //   scan(b)   exclusive prefix over the counts: bin offsets (counting sort).
