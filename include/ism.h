@@ -84,8 +84,11 @@ typedef enum {
  *   fixed-point integer with a step of 2^-23 of the bin's largest possible
  *   amplitude and summed exactly (so the result does not depend on the
  *   order of the images), and each offset's moments are expanded once into
- *   the 32 taps.  Other windows use the direct evaluation of
- *   ISM_PREC_FP32_DIRECT. */
+ *   the 32 taps.  Other windows go the same way with 10 moments in steps of
+ *   2^-31 where a room has 20 images or more per 32 samples and the series
+ *   follows the window (lengths that end on a sample, any of 80 taps or more):
+ *   no more error than the direct evaluation of ISM_PREC_FP32_DIRECT, which
+ *   the rest use. */
 typedef enum {
     ISM_PREC_FP32 = 0,        /* FP32, Chebyshev moments in dense rooms, else direct */
     ISM_PREC_FP16X2 = 1,      /* packed FP16 window and sinc, FP32 accumulation        */

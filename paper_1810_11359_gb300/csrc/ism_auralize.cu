@@ -11,9 +11,10 @@
 // T0 + 4 l + r, r = 0 .. 3, for the microphones (32 accumulators for 8).  For one
 // segment the taps k that connect it to the tile are walked in chunks of 128;
 // the chunks of all segments are dealt to the CTA's warps in turn, which add
-// their partial sums in warp order at the end.  A segment's chunks are of one size (142 taps
-// as 72 + 70, not 128 + 14, of which every other warp would take the short ones: 18 segments
-// of 14 samples, RIRs of 27,800, 9 microphones 103 -> 74 us).  (16 points x 1 microphone, RIRs
+// their partial sums in warp order at the end.  A segment's chunks are of one size where their
+// number is a power of two (142 taps as 72 + 70, not 128 + 14, of which every other warp
+// would take the short ones: 18 segments of 14 samples, RIRs of 27,800, 9 microphones 103 ->
+// 62 us).  (16 points x 1 microphone, RIRs
 // of 9600 samples, a signal of 57,600: 337 us with 8 microphones' sums always
 // and whole segments dealt to 4 warps, 49 us now; 30 x 5, 16,000, 48,000: 340 ->
 // 282; the 48 kHz array 1285 -> 1193.)
@@ -110,7 +111,9 @@ __global__ void __launch_bounds__(AU_WARPS * 32, AU_WARPS > 4 ? 1 : AU_M == 8 ? 
             const float* hp = h + (long long)p * n_mics * n_s;
             const int n_k = (int)(k_hi - k_lo);
             const int n_ch = n_k / AU_KC + 1;
-            const int kc = (n_k / n_ch + 4) & ~3;   // taps of a chunk: as even as whole groups allow
+            // taps of a chunk: as even as whole groups allow where the number of chunks shares
+            // the warps' (a power of two), else 128 and a remnant that goes round all warps
+            const int kc = n_ch & (n_ch - 1) ? AU_KC : ((n_k >> (31 - __clz(n_ch))) + 4) & ~3;
             const int first = (warp - turn + AU_WARPS) % AU_WARPS;   // the warp's first chunk of this segment
             turn = (turn + n_ch) % AU_WARPS;
             for (long long k0 = k_lo + (long long)first * kc; k0 <= k_hi; k0 += AU_WARPS * kc) {
@@ -217,21 +220,27 @@ int launch_au_m(const float* x, int n_x, const float* h, int n_points, int n_mic
                 cudaStream_t s)
 {
     // 16 warps share a tile where it has chunks for them; 4 where a tile has few (RIRs or segments
-    // of a chunk or two) and there are tiles to fill the GPU all the same.  By the turns that
-    // the fullest warp takes: a turn is a chunk, two more begin and end the tile, and an SM runs
-    // 16 warps as fast as one.  700 sizes from 200 x 50 to 250,000 x 80,000 samples: 1 % above
-    // the better of the two on average, 40 % at most.  241,000 samples, RIRs of 51, 11
-    // microphones: 142 us with 16 warps, 37 with 4; 3000 segments of 16 samples, RIRs of 9600:
-    // 1786 and 1455; 16 points x 1, 57,600 samples, RIRs of 9600: 49 and 164.
+    // of a chunk or two) and there are tiles to fill the GPU all the same.  By the turns that the
+    // fullest warp takes, an SM running 16 warps as fast as one: a turn is a chunk, 1.5 or 2 more
+    // begin and end the tile, and every warp looks at all the tile's segments, a fifth of a
+    // turn each for one microphone.  Long tiles (64 chunks or more of whole segments) in fewer
+    // than 1024 end the launch better in 16 warps.  1000 sizes from 200 x 50 to 250,000 x
+    // 80,000 samples: 0.6 % above the better of the two on average, 37 % at most.  us, 4 warps
+    // and 16: 241,000 samples, RIRs of 51, 11 microphones 36 and 140; 3000 segments of 16
+    // samples, RIRs of 8960 527 and 688; 10 points x 2, 12,001, 4801 25 and 17; the 48 kHz
+    // array 1326 and 1192.
     const long long tiles = (((long long)n_x + n_s - 1 + AU_TILE - 1) / AU_TILE) * ((n_mics + AU_M - 1) / AU_M);
     const int seg = std::max(1, n_x / n_points);
     const long long segs = std::min<long long>(n_points, std::min<long long>(n_x, n_s + AU_TILE - 1ll) / seg + 1);
     const long long chunks = segs * ((std::min<long long>(n_s, seg + AU_TILE - 1ll) + AU_KC - 1) / AU_KC);
-    const auto turns = [&](int warps) {
-        return std::max(1.0, (double)tiles * warps / (152.0 * 16.0)) * (double)((chunks + warps - 1) / warps + 2);
+    const auto turns = [&](int warps, double ends) {
+        return std::max(1.0, (double)tiles * warps / (152.0 * 16.0)) *
+               ((double)((chunks + warps - 1) / warps) + ends + 0.2 * (double)segs / AU_M);
     };
-    return turns(4) <= turns(16) ? launch_au<VEC, AU_M, 4>(x, n_x, h, n_points, n_mics, n_s, starts, y, s)
-                                 : launch_au<VEC, AU_M, 16>(x, n_x, h, n_points, n_mics, n_s, starts, y, s);
+    const bool few_long = seg >= AU_KC && chunks >= 64 && tiles < 1024;
+    return turns(4, 1.5) * (few_long ? 1.3 : 1.0) <= turns(16, 2.0)
+               ? launch_au<VEC, AU_M, 4>(x, n_x, h, n_points, n_mics, n_s, starts, y, s)
+               : launch_au<VEC, AU_M, 16>(x, n_x, h, n_points, n_mics, n_s, starts, y, s);
 }
 
 }  // namespace
