@@ -63,7 +63,7 @@
 #define ISM_CHEB_TAB_CTAS 32      // CTAs that fill one (8 taps each)
 #define ISM_SHELL_BINS 8          // delay bins per CTA of the fused Chebyshev accumulation
 #define ISM_SD_BINS 32            // delay bins per CTA of the fused direct accumulation
-#define ISM_SPLIT_SAMPLES 22600   // n_ism + H up to which FP32 jobs split their squared offsets (ism_shell.cuh)
+#define ISM_SPLIT_SAMPLES 15980   // n_ism + H up to which FP32 jobs split their squared offsets (ism_shell.cuh)
 #define ISM_FILL_CTAS 304         // fused CTAs a launch set should have at least (two per SM of a GB300)
 #define ISM_WAVE_CTAS 760         // fused CTAs that run at once (five per SM)
 #define ISM_THIN_IMAGES 3500.0    // images per fused CTA from which thinner shells balance a single wave

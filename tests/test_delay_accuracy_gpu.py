@@ -22,7 +22,7 @@ N_SRC = 96
 K = FS / float(np.float32(C))
 ROUNDED = 3e-8 + 2e-7 / 1.81
 # on both sides of the length from which the offsets are no longer split, and the longest
-LENGTHS = [9600, 22500, 22700, 57600, 131000]
+LENGTHS = [9600, 15900, 16000, 22500, 22700, 57600, 131000]
 
 
 @pytest.fixture(scope="module", autouse=True)
