@@ -1666,11 +1666,9 @@ ism_status ism_auralize(const float* signal, int n_x, const float* rirs, int n_p
 // The form that ism_auralize_ex takes (an ism_auralize_form), from the sizes alone, with the
 // plans: *af with the default chunk (of *af_need bytes of workspace), *ao.  -1: the FFT form
 // is asked for an output too long for it.
-// The automatic choice compares times estimated at measured rates.  Four-step against
-// direct: about 4 N log2 N lane operations per length-N DFT (one per segment, one per
-// microphone pair and point, one inverse per pair) and 4 per product of spectra (8.0 T/s)
-// against n_mics n_x n_S multiply-adds (20.5 T/s).  Overlap-save, where its plan exists,
-// as the plan says, against the multiply-adds of the direct form with microphones
+// The automatic choice compares times estimated at measured rates: an FFT form's (the plan's,
+// or the four-step form's, whose lane operations also have to be below 1 / 2.55 of the n_mics
+// n_x n_S multiply-adds) against the multiply-adds of the direct form with microphones
 // padded to 1, 2, 4 or 8 a CTA and a segment's taps to whole chunks of 128 for every tile of
 // 128 outputs (17 T/s of them, 1 microphone 11; 5 us).  Over 410 sizes the choice takes 0.4 %
 // more than the better of the two on average, 37 % at most.  Direct and overlap-save, us:
@@ -1691,17 +1689,20 @@ static int auralize_form(int n_x, int n_points, int n_mics, int n_S, bool unifor
     const bool ols = ism_auralize_ols_plan(n_x, n_points, n_mics, n_S, uniform, af->logN, least, ao);
     const int fft_form = ols ? ISM_AURALIZE_FORM_OVERLAP_SAVE : ISM_AURALIZE_FORM_FOUR_STEP;
     if (method == ISM_AURALIZE_FFT) return fft_form;
-    const double N = (double)af->N, pairs = (double)af->n_pairs;
-    const double fft =
-        ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * af->logN + (double)n_points * pairs * 4.0 * N;
-    const double direct = (double)n_mics * (double)n_x * (double)n_S;
-    if (!ols) return direct > 2.55 * fft ? ISM_AURALIZE_FORM_FOUR_STEP : ISM_AURALIZE_FORM_DIRECT;
     const double len = (double)n_x / n_points;
     const double padded = std::ceil((len + 127.0) / 128.0) * 128.0 / len;
     const int mics = n_mics <= 2 ? n_mics : n_mics <= 4 ? 4 : (n_mics + 7) / 8 * 8;
     const double issued = (double)mics * (double)n_x * (double)n_S * padded;
-    return 5.0e-6 + issued / (mics == 1 ? 1.1e13 : 1.7e13) > ao->seconds ? ISM_AURALIZE_FORM_OVERLAP_SAVE
-                                                                        : ISM_AURALIZE_FORM_DIRECT;
+    const double direct = 5.0e-6 + issued / (mics == 1 ? 1.1e13 : 1.7e13);
+    if (ols) return direct > ao->seconds ? ISM_AURALIZE_FORM_OVERLAP_SAVE : ISM_AURALIZE_FORM_DIRECT;
+    // (four-step: only where its operations speak for it too)
+    const double N = (double)af->N, pairs = (double)af->n_pairs;
+    const double ops =
+        ((double)n_points * (1.0 + pairs) + pairs) * 4.0 * N * af->logN + (double)n_points * pairs * 4.0 * N;
+    return (double)n_mics * (double)n_x * (double)n_S > 2.55 * ops &&
+                   direct > ism_auralize_four_step_seconds(af->logN, n_points, af->n_pairs)
+               ? ISM_AURALIZE_FORM_FOUR_STEP
+               : ISM_AURALIZE_FORM_DIRECT;
 }
 
 static ism_status auralize_args(const float* signal, int n_x, const float* rirs, int n_points, int n_mics, int n_S,

@@ -393,6 +393,15 @@ static bool ao_sizes(int n_x, int P, int M, int n_S, bool uniform, AoPlan& pl, d
     return true;
 }
 
+// Seconds of the four-step form, roughly: its launches, and per length-N DFT (one per segment,
+// one per microphone pair and point, one inverse per pair) 4 N log2 N lane operations and 4 N
+// per product of spectra, at 6 T/s.
+double ism_auralize_four_step_seconds(int logN, int P, int pairs)
+{
+    const double N = (double)(1ll << logN);
+    return 2.4e-5 + (((double)P * (1.0 + pairs) + pairs) * 4.0 * N * logN + (double)P * pairs * 4.0 * N) / 6.0e12;
+}
+
 // Whether the overlap-save form takes a filtering, and its plan.  It does where its DFTs'
 // operations are below 1.3 times the four-step form's (one DFT of 2^logN per segment and
 // per (point, pair)), which passes over device memory twice.  Measured at a ratio of 0.35
@@ -433,9 +442,13 @@ bool ism_auralize_ols_plan(int n_x, int P, int M, int n_S, bool uniform, int log
         if (off <= ws_min) break;
         if (pl.G == 1) return false;
     }
-    const double pieces = (uniform ? (double)P * pl.cuts : 1.3 * P) * std::min(1.0, ((double)n_S + pl.V) / n_x);
+    const double pieces = (uniform ? (double)P * pl.cuts : std::min(1.3 * P, (double)n_x)) *
+                          std::min(1.0, ((double)n_S + pl.V) / n_x);
     const double ctas = (double)units * pl.G;
     pl.seconds = 2.6e-5 + std::max(flops / 1.4e13, std::ceil(pieces / pl.G) * 2.0e-6 * std::max(1.0, ctas / 304.0));
+    // (nor where a chain of pieces makes it longer than the four-step form: 44 segments of 7
+    // samples x 3 microphones, RIRs of 6720, 136 and 38 us)
+    if (pl.seconds > 1.15 * ism_auralize_four_step_seconds(logN, P, pl.n_pairs)) return false;
     *out = pl;
     return true;
 }

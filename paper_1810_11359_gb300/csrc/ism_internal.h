@@ -278,6 +278,7 @@ int ism_launch_auralize(const float* x, int n_x, const float* h, int n_points, i
 int ism_auralize_fft_plan(int n_x, int n_points, int n_mics, int n_S, size_t ws_bytes, AfPlan* out, size_t* need);
 int ism_launch_auralize_fft(const float* x, const float* h, const int* starts, float* y, const AfPlan& pl, char* ws,
                             void* stream);
+double ism_auralize_four_step_seconds(int logN, int P, int pairs);
 bool ism_auralize_ols_plan(int n_x, int n_points, int n_mics, int n_S, bool uniform, int logN, size_t ws_min,
                            AoPlan* out);
 int ism_launch_auralize_ols(const float* x, const float* h, const int* starts, float* y, const AoPlan& pl, char* ws,

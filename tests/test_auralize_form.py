@@ -69,6 +69,15 @@ def test_automatic_choice_counts_the_pieces_that_follow_one_another(size, given,
     assert ism.ism_auralize_form(*size, given_starts=given) == form
 
 
+@pytest.mark.parametrize("size,given,form", [
+    ((312, 44, 3, 6720), True, "four_step"),       # 44 pieces in turn take longer than its passes
+    ((387, 107, 15, 2477), False, "four_step"),
+    ((100, 100, 8, 9000), False, "overlap_save"),  # the passes longer still
+    ((57600, 64, 8, 57600), False, "overlap_save")])
+def test_fft_method_takes_the_faster_form(size, given, form):
+    assert ism.ism_auralize_form(*size, method="fft", given_starts=given) == form
+
+
 @pytest.mark.parametrize("size", [(57600, 64, 8, 57600), (57600, 64, 2, 4800), (30000, 64, 4, 3200), (144000, 500, 2, 19200)])
 def test_workspace_of_the_overlap_save_form(size):
     """The automatic choice asks for the overlap-save form's piece spectra (18 KB each; of given
