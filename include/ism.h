@@ -86,7 +86,7 @@ typedef enum {
  *   order of the images), and each offset's moments are expanded once into
  *   the 32 taps.  Other windows go the same way with 10 moments in steps of
  *   2^-31 where a room has 20 images or more per 32 samples and the series
- *   follows the window (lengths that end on a sample, any of 80 taps or more):
+ *   follows the window (lengths that end on a sample, any of 47 taps or more):
  *   no more error than the direct evaluation of ISM_PREC_FP32_DIRECT, which
  *   the rest use. */
 typedef enum {

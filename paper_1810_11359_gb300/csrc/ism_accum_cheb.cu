@@ -62,7 +62,7 @@
 // A window whose end falls inside a sample interval cuts its last taps with a
 // mask, which no polynomial follows, but the window has a double zero there:
 // the kink falls with the cube of the window's length, and degree 9 reproduces the
-// taps to 2.6e-8 of the amplitude (1e-8 without a mask; norms over the taps) for the
+// taps to 4.5e-8 of the amplitude (5e-9 without a mask; rms, norms over the taps) for the
 // windows that this form takes (series_follows_window).  The 2 H coefficients
 // of each term come from a table in the workspace that the geometry launch
 // fills (cheb_table), and the expansion takes 32 taps at a time, each turn's

@@ -179,15 +179,15 @@ double images_in_reach(const Validated& v)
 // job's window (other than 32 taps).  A window that ends inside a sample interval, theta of
 // it, cuts its outermost taps there; what the series of degree 9 misses of them is at most
 // 0.018 sin(pi theta) / N_w^3 of an image's amplitude (norm over the taps; every N_w from 16 to
-// 256 in steps of 0.1), where the FP32 rounding of a tap-by-tap sum leaves about 1.1e-7.  The
-// rule admits 2.6e-8 of it: windows that end on a sample, any from 80 taps on, and those
-// between that end close to a sample (44.1 taps).  Relative error of RIRs of 17.5,
-// 20.8, 24.8 and 33.3 taps: 3.2, 3.7, 2.4 and 1.4e-7 through the series, 1.0 to 1.1e-7 tap by
-// tap, the form that they take.
+// 256 in steps of 0.1), rms a quarter of that.  The rule admits windows that end on a sample, any from 46.4
+// taps on (rms 4.5e-8), and those between that end close to a sample (44.1 taps): over 20
+// windows of 46.5 to 79 taps the RIRs' error through the series is 0.96 of the tap-by-tap
+// sum's (1.2e-7 of the norm).  Relative error of RIRs of 17.5, 20.8, 24.8 and 33.3 taps: 3.2,
+// 3.7, 2.4 and 1.4e-7 through the series, 1.0 to 1.1e-7 tap by tap, the form that they take.
 bool series_follows_window(const Validated& v)
 {
     const double theta = 0.5 * v.Nw - (v.H - 1);   // in (0, 1]
-    return v.Nw >= ISM_CHEB_MIN_NW && v.Nw * v.Nw * v.Nw >= 5.0e5 * std::sin(M_PI * theta);
+    return v.Nw >= ISM_CHEB_MIN_NW && v.Nw * v.Nw * v.Nw >= 1.0e5 * std::sin(M_PI * theta);
 }
 
 // Lays the launch set out in the workspace from byte offset `base` on (the

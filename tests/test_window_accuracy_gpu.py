@@ -46,6 +46,13 @@ def test_dense_windows(taps):
     assert np.sqrt(np.mean(_errors(taps, "fp32") ** 2)) <= 2e-7
 
 
+def test_cut_windows_have_no_more_error_than_the_taps_one_by_one():
+    """The shortest windows that end inside a sample interval and go through the series."""
+    taps = [46.5, 47.0, 47.7, 48.6, 49.0, 50.7, 51.3, 53.0, 55.5, 57.4, 60.3, 61.0, 63.2, 65.0, 67.7, 70.4, 73.0, 75.1, 77.0, 79.0]
+    series, direct = (np.concatenate([_errors(t, p, 8) for t in taps]) for p in ("fp32", "fp32_direct"))
+    assert np.mean(series ** 2) <= np.mean(direct ** 2)
+
+
 def test_series_has_no_more_error_than_the_taps_one_by_one():
     """Windows that go through the series, over lengths whose rounded coefficients differ."""
     taps = [16.0, 18.0, 24.0, 36.0, 44.0, 50.0, 64.0, 82.5, 88.2, 96.7, 110.25, 128.0, 150.3, 176.4, 192.0, 224.5]
